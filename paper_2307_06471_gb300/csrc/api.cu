@@ -182,13 +182,16 @@ int default_launch(crkdg_ctx* c) {
     return wave_rows(c, c->wpb, 1, &c->seg_rows);
 }
 
-int enqueue_reduce(crkdg_ctx* c, int set_dt) {
-    const int blocks = 4 * std::max(1, crk::sm_count());
-    int r = ensure_partials(c, (size_t)blocks * 8 * 8);
+// the FP64 reduction of the current averages: the maximum wave speed, and what
+// `run` asks for
+int enqueue_reduce(crkdg_ctx* c, crk::ReduceRun run) {
+    run.set_estimate(c->gamma, dx_of(c), dy_of(c));
+    const int blocks = crk::reduce_blocks(c->ncell, crk::sm_count());
+    int r = ensure_partials(c, (size_t)blocks * crk::REDUCE_SLOT);
     if (r) return r;
     CK(crk::launch_reduce(c->dim, c->kphys, c->precision, c->u[c->cur], c->mesh.nx, c->dim == 1 ? 1 : c->mesh.ny, c->nm,
                           dx_of(c), dy_of(c), c->gamma, c->beta[0], c->beta[1], c->d_state, c->d_partials, blocks,
-                          set_dt, c->stream));
+                          run, c->stream));
     return CRKDG_OK;
 }
 
@@ -341,11 +344,6 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
 }
 
 int check_ctx(const crkdg_ctx* c) { return c ? CRKDG_OK : fail(CRKDG_EINVAL, "null context"); }
-
-__global__ void set_run_params(DevState* ds, double cfl, double t_end) {
-    ds->cfl = cfl;
-    ds->t_end = t_end;
-}
 
 }  // namespace
 
@@ -653,7 +651,7 @@ int crkdg_get_state(crkdg_ctx* c, double* h) {
 int crkdg_cfl_dt(crkdg_ctx* c, double cfl, double* dt_out) {
     if (check_ctx(c) || !dt_out) return fail(CRKDG_EINVAL, "null argument");
     if (!(cfl > 0.0)) return fail(CRKDG_EINVAL, "cfl must be positive");
-    int r = enqueue_reduce(c, 0);
+    int r = enqueue_reduce(c, {0, 0, 0.0, 0.0});
     if (r) return r;
     double ms = 0.0;
     CK(cudaMemcpyAsync(&ms, &c->d_state->maxspeed, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -688,9 +686,7 @@ int crkdg_advance(crkdg_ctx* c, int n_steps, double cfl, double t_end, int captu
     if (!(cfl > 0.0)) return fail(CRKDG_EINVAL, "cfl must be positive");
     if (n_steps == 0) return CRKDG_OK;
     // run parameters and the first dt from the current state
-    set_run_params<<<1, 1, 0, c->stream>>>(c->d_state, cfl, t_end);
-    CK(cudaGetLastError());
-    int r = enqueue_reduce(c, 1);
+    int r = enqueue_reduce(c, {0, 1, cfl, t_end});
     if (r) return r;
     const int lim_first = c->pending ? 1 : 0;
     const int lim_rest = (c->limiter_on || c->pp_eps > 0.0) ? 1 : 0;
@@ -960,7 +956,7 @@ int crkdg_features(crkdg_ctx* c, float* X_dev, float* y_dev, double M) {
 
 int crkdg_conservation(crkdg_ctx* c, double* sums) {
     if (check_ctx(c) || !sums) return fail(CRKDG_EINVAL, "null argument");
-    int r = enqueue_reduce(c, 0);
+    int r = enqueue_reduce(c, {1, 0, 0.0, 0.0});
     if (r) return r;
     CK(cudaMemcpyAsync(sums, c->d_state->sums, c->nv * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -1136,7 +1132,7 @@ int crkdg_autotune(crkdg_ctx* c, double* best_us) {
     const int cur0 = c->cur;
     double dt = 0.0;
     {
-        int r = enqueue_reduce(c, 0);
+        int r = enqueue_reduce(c, {0, 0, 0.0, 0.0});
         if (r) return r;
         double ms = 0.0;
         CK(cudaMemcpy(&ms, &c->d_state->maxspeed, sizeof(double), cudaMemcpyDeviceToHost));

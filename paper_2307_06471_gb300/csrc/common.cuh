@@ -31,6 +31,30 @@ struct DevState {
     unsigned long long lim_count;   // cells flagged by a separate limiter pass since the last step
 };
 
+// The reduction of a state's averages (reduce_state_kernel): what it does
+// beside the maximum wave speed
+struct ReduceRun {
+    int want_sums;        // the totals too
+    int set_dt;           // start of a device-driven run: store cfl and t_end, dt = min(cfl / max, t_end - t)
+    double cfl, t_end;
+    float gammaf = 0.f, rxf = 0.f, ryf = 0.f;   // FP32 gamma, 1/dx, 1/dy of the estimates (set_estimate)
+    void set_estimate(double gamma, double dx, double dy) {
+        gammaf = (float)gamma;
+        rxf = (float)(1.0 / dx);
+        ryf = (float)(1.0 / dy);
+    }
+};
+
+constexpr int REDUCE_THREADS = 256;
+constexpr int REDUCE_CPT = 4;   // cells per thread in flight
+constexpr size_t REDUCE_SLOT = 6;   // doubles per block of its scratch
+// Blocks of a reduction over `cells` cells: one chunk each, at most four per SM
+inline int reduce_blocks(size_t cells, int sms) {
+    const size_t chunk = (size_t)REDUCE_THREADS * REDUCE_CPT;
+    const size_t n = (cells + chunk - 1) / chunk, most = (size_t)4 * (sms > 0 ? sms : 1);
+    return (int)(n < 1 ? 1 : (n < most ? n : most));
+}
+
 struct BCSide {
     int type;
     int fn;
@@ -457,6 +481,13 @@ __device__ __forceinline__ float opaque(float v) {
 __device__ __forceinline__ double opaque(double v) {
     asm volatile("" : "+d"(v));
     return v;
+}
+
+// a wave speed as an ordered key: NaN (ignored, as fmax does) and -0 map to 0
+__device__ __forceinline__ unsigned long long speed_key(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const bool neg = b >> 63, nan = (b & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+    return neg || nan ? 0ull : b;
 }
 
 // f(std::integral_constant<int, i>) for i = 0 .. N-1: loops whose index must

@@ -76,9 +76,9 @@ cudaError_t project1d_k(int k, const double* vals, void* u, int ncell, cudaStrea
 
 template <class T, int PHYS, int NV>
 cudaError_t reduce_t(const void* u, int nx, int ny, int nm, double dx, double dy, double gamma, double bx,
-                     double by, DevState* ds, double* partials, int blocks, int set_dt, cudaStream_t st) {
-    reduce_state_kernel<T, PHYS, NV><<<blocks, 256, 0, st>>>(static_cast<const T*>(u), nx, ny, nm, dx, dy, gamma,
-                                                              bx, by, ds, partials, set_dt);
+                     double by, DevState* ds, double* partials, int blocks, const ReduceRun& run, cudaStream_t st) {
+    reduce_state_kernel<T, PHYS, NV><<<blocks, REDUCE_THREADS, 0, st>>>(static_cast<const T*>(u), nx, ny, nm, dx, dy, gamma,
+                                                              bx, by, ds, partials, run);
     return cudaGetLastError();
 }
 
@@ -100,10 +100,10 @@ cudaError_t info_step1d(int phys, int prec, int k, int s, KernelInfo* info) {
 }
 
 cudaError_t launch_reduce(int dim, int phys, int prec, const void* u, int nx, int ny, int nm, double dx, double dy,
-                          double gamma, double bx, double by, DevState* ds, double* partials, int blocks, int set_dt,
-                          cudaStream_t st) {
-    if (prec == 2 || prec == 3) return reduce_euler_f32c(u, nx, ny, nm, dx, dy, gamma, ds, partials, blocks, set_dt, st);
-#define CRK_R(T, P, NV) reduce_t<T, P, NV>(u, nx, ny, nm, dx, dy, gamma, bx, by, ds, partials, blocks, set_dt, st)
+                          double gamma, double bx, double by, DevState* ds, double* partials, int blocks,
+                          const ReduceRun& run, cudaStream_t st) {
+    if (prec == 2 || prec == 3) return reduce_euler_f32c(u, nx, ny, nm, dx, dy, gamma, ds, partials, blocks, run, st);
+#define CRK_R(T, P, NV) reduce_t<T, P, NV>(u, nx, ny, nm, dx, dy, gamma, bx, by, ds, partials, blocks, run, st)
     if (phys == PHYS_ADV) return prec == 0 ? CRK_R(float, PHYS_ADV, 1) : CRK_R(double, PHYS_ADV, 1);
     if (dim == 1) return prec == 0 ? CRK_R(float, PHYS_EULER1D, 3) : CRK_R(double, PHYS_EULER1D, 3);
     return prec == 0 ? CRK_R(float, PHYS_EULER, 4) : CRK_R(double, PHYS_EULER, 4);

@@ -70,9 +70,9 @@ cudaError_t project2d_euler_f32c(int k, int basis, const double* vals, void* u, 
     CRK_SWITCH(run_project_c, vals, u, ncell, st)
 }
 cudaError_t reduce_euler_f32c(const void* u, int nx, int ny, int nm, double dx, double dy, double gamma, DevState* ds,
-                              double* partials, int blocks, int set_dt, cudaStream_t st) {
-    reduce_state_kernel<float, PHYS_EULER, 4, true><<<blocks, 256, 0, st>>>(
-        static_cast<const float*>(u), nx, ny, nm, dx, dy, gamma, 0.0, 0.0, ds, partials, set_dt);
+                              double* partials, int blocks, const ReduceRun& run, cudaStream_t st) {
+    reduce_state_kernel<float, PHYS_EULER, 4, true><<<blocks, REDUCE_THREADS, 0, st>>>(
+        static_cast<const float*>(u), nx, ny, nm, dx, dy, gamma, 0.0, 0.0, ds, partials, run);
     return cudaGetLastError();
 }
 

@@ -42,10 +42,11 @@ cudaError_t launch_project(int dim, int phys, int prec, int k, int basis, const 
 cudaError_t launch_step1d(int phys, int prec, int k, const StepArgs& a, int n_steps, int threads, int blocks,
                           cudaStream_t st);
 cudaError_t info_step1d(int phys, int prec, int k, int s, KernelInfo* info);
-// FP64 reduction of the averages into DevState (set_dt: also dt = cfl/max)
+// FP64 reduction of the averages into DevState (aux_kernels.cuh); partials
+// holds REDUCE_SLOT doubles per block
 cudaError_t launch_reduce(int dim, int phys, int prec, const void* u, int nx, int ny, int nm, double dx, double dy,
-                          double gamma, double bx, double by, DevState* ds, double* partials, int blocks, int set_dt,
-                          cudaStream_t st);
+                          double gamma, double bx, double by, DevState* ds, double* partials, int blocks,
+                          const ReduceRun& run, cudaStream_t st);
 
 // per-(phys, prec) entry points defined in the kernel translation units
 #define CRK_DECL_2D(NAME)                                                                                  \
@@ -59,7 +60,7 @@ cudaError_t step2d_euler_f32c(int k, int basis, const StepArgs& a, int wpb, cuda
 cudaError_t info2d_euler_f32c(int k, int basis, int s, KernelInfo* info);
 cudaError_t project2d_euler_f32c(int k, int basis, const double* vals, void* u, int ncell, cudaStream_t st);
 cudaError_t reduce_euler_f32c(const void* u, int nx, int ny, int nm, double dx, double dy, double gamma, DevState* ds,
-                              double* partials, int blocks, int set_dt, cudaStream_t st);
+                              double* partials, int blocks, const ReduceRun& run, cudaStream_t st);
 
 // compensated FP32 state with deviation-form fluxes (same planes as f32c)
 cudaError_t step2d_euler_f32d(int k, int basis, const StepArgs& a, int wpb, cudaStream_t st);

@@ -110,11 +110,13 @@ extern "C" int crkdg_reduce_state_noalloc(const void* u_dev, int dim, int nx, in
     if (e != cudaSuccess) return fail(CRKDG_ECUDA, std::string("clearing scratch: ") + cudaGetErrorString(e));
     const double bx = beta ? beta[0] : 0.0, by = beta && dim == 2 ? beta[1] : 0.0;
     const int kphys = physics == CRKDG_ADVECTION ? crk::PHYS_ADV : (dim == 1 ? crk::PHYS_EULER1D : crk::PHYS_EULER);
+    crk::ReduceRun run{1, 0, 0.0, 0.0};
+    run.set_estimate(gamma, dx, dy);
     int nv = 1;
 #define CRK_NA(T, P, NV)                                                                                     \
     crk::reduce_state_kernel<T, P, NV><<<kNoAllocBlocks, 256, 0, st>>>(static_cast<const T*>(u_dev), nx, ny,  \
                                                                       n_modes, dx, dy, gamma, bx, by, &s->ds, \
-                                                                      s->partials, 0);                       \
+                                                                      s->partials, run);                      \
     nv = NV;
     if (kphys == crk::PHYS_ADV) {
         if (precision == CRKDG_F32) { CRK_NA(float, crk::PHYS_ADV, 1) } else { CRK_NA(double, crk::PHYS_ADV, 1) }

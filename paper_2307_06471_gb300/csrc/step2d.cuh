@@ -313,13 +313,6 @@ __device__ __forceinline__ void step_epilogue(const StepArgs& a, const PV& pv, i
 // and the troubled count is an integer.
 constexpr int FINALIZE_THREADS = 256;
 
-// a slot's speed as an ordered key: NaN (ignored, as fmax does) and -0 map to 0
-__device__ __forceinline__ unsigned long long speed_key(double v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const bool neg = b >> 63, nan = (b & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
-    return neg || nan ? 0ull : b;
-}
-
 template <int NV>
 __global__ void __launch_bounds__(FINALIZE_THREADS) finalize_step_kernel(const StepArgs a, int total_warps) {
     constexpr int NRED = NV + 2;
