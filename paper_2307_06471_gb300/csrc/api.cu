@@ -62,6 +62,8 @@ struct crkdg_ctx {
     DevState* d_state;
     double* d_partials;
     size_t partials_cap;
+    void* d_seam = nullptr;       // seam scratch of the 2D step
+    size_t seam_cap = 0;          // its bytes
     unsigned long long* d_flags;
     cudaStream_t stream;
     double t;
@@ -132,12 +134,51 @@ void strips_segs(const crkdg_ctx* c, int seg_rows, int* ns, int* nseg) {
     *nseg = (c->mesh.ny + seg_rows - 1) / seg_rows;
 }
 
+// bytes of one segment's seam scratch (2D quadrature step)
+size_t seam_seg_bytes(const crkdg_ctx* c) {
+    return crk::seam_values(c->tab.s, c->k + 1, c->nv, c->nm, c->precision == CRKDG_F32D,
+                            c->limit_mode == CRKDG_LIMIT_FUSED, c->mesh.nx) * c->esize;
+}
+// whether the quadrature step leaves the faces between its segments to the
+// seam launches (the compensated state without
+// deviation fluxes recomputes halo rows)
+bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load) {
+    return c->precision != CRKDG_F32C && crk::use_seams(c->esize, c->tab.s, c->nm, lim_on_load, c->mesh.ny, nseg);
+}
+
+// launch geometry of the quadrature step (its scratch bounds the segments)
+void step_segs(const crkdg_ctx* c, int* ns, int* nseg) {
+    strips_segs(c, c->seg_rows, ns, nseg);
+    if (step_seams(c, *nseg, false))
+        *nseg = crk::seam_segments(*nseg, seam_seg_bytes(c), c->elems * c->esize * c->planes);
+}
+
 int ensure_partials(crkdg_ctx* c, size_t n) {
     if (n <= c->partials_cap) return CRKDG_OK;
     if (c->d_partials) cudaFree(c->d_partials);
     c->d_partials = nullptr;
     CK(cudaMalloc(&c->d_partials, n * sizeof(double)));
     c->partials_cap = n;
+    return CRKDG_OK;
+}
+
+// the quadrature step's scratch: reduction slots and seams
+int ensure_step_scratch(crkdg_ctx* c) {
+    int ns, nseg;
+    step_segs(c, &ns, &nseg);
+    int r = ensure_partials(c, ((size_t)ns * nseg + crk::seam_blocks(c->nv, c->mesh.nx, c->mesh.ny, nseg, 2 * std::max(1, crk::sm_count()))) * (c->nv + 2));
+    if (r) return r;
+    const size_t need = step_seams(c, nseg, false) ? seam_seg_bytes(c) * nseg : 0;
+    if (need <= c->seam_cap) return CRKDG_OK;
+    if (c->d_seam) cudaFree(c->d_seam);
+    c->d_seam = nullptr;
+    c->seam_cap = 0;
+    if (cudaMalloc(&c->d_seam, need) != cudaSuccess) {
+        cudaGetLastError();
+        c->d_seam = nullptr;
+        return fail(CRKDG_ENOMEM, "cudaMalloc of the step's seam scratch failed");
+    }
+    c->seam_cap = need;
     return CRKDG_OK;
 }
 
@@ -179,7 +220,15 @@ int default_launch(crkdg_ctx* c) {
     if (w < 0) return w;
     c->wpb = std::min(w, 4);
     // one wave: as many warps as the SMs hold at once
-    return wave_rows(c, c->wpb, 1, &c->seg_rows);
+    int r = wave_rows(c, c->wpb, 1, &c->seg_rows);
+    if (r) return r;
+    // a mesh with fewer warps than that: blocks small enough to reach every SM
+    // (the FP64 vortex at 80^2 has 240 warps: 0.284 ms a step in blocks of 4,
+    // 0.243 ms in blocks of 1)
+    int ns, nseg;
+    step_segs(c, &ns, &nseg);
+    while (c->wpb > 1 && (long)ns * nseg < (long)c->wpb * crk::sm_count()) c->wpb /= 2;
+    return CRKDG_OK;
 }
 
 // the FP64 reduction of the current averages: the maximum wave speed, and what
@@ -279,13 +328,15 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
     a.pp_eps = limit ? c->pp_pending : 0.0;
     if (c->dim == 2) {
         int ns, nseg;
-        strips_segs(c, c->seg_rows, &ns, &nseg);
+        step_segs(c, &ns, &nseg);
         a.seg_len = c->seg_rows;
         a.n_strips = ns;
         a.n_segs = nseg;
-        int r = ensure_partials(c, (size_t)ns * nseg * 8);
+        int r = ensure_step_scratch(c);
         if (r) return r;
         a.partials = c->d_partials;
+        a.seam = c->d_seam;
+        a.seams = step_seams(c, nseg, a.limit && c->limit_mode == CRKDG_LIMIT_FUSED);
         if (c->mlp && limit && M >= 0.0 && c->limit_mode == CRKDG_LIMIT_FUSED) {
             a.mlp = c->mlp;
             a.mlp_zlo = c->mlp_zlo;
@@ -465,6 +516,10 @@ int create_impl(const crkdg_mesh* mesh, int k, int basis, int flux, const crkdg_
     if (r) return bail(r);
     r = default_launch(c);
     if (r) return bail(r);
+    if (c->dim == 2 && !use_linear(c)) {   // a step allocates nothing
+        r = ensure_step_scratch(c);
+        if (r) return bail(r);
+    }
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return bail(fail(CRKDG_ECUDA, "stream sync failed"));
     *out = c;
     return CRKDG_OK;
@@ -540,6 +595,7 @@ void crkdg_destroy(crkdg_ctx* c) {
     if (c->d_tab) cudaFree(c->d_tab);
     if (c->d_state) cudaFree(c->d_state);
     if (c->d_partials) cudaFree(c->d_partials);
+    if (c->d_seam) cudaFree(c->d_seam);
     if (c->d_flags) cudaFree(c->d_flags);
     if (c->u3) cudaFree(c->u3);
     if (c->d_stage) cudaFree(c->d_stage);
@@ -692,13 +748,12 @@ int crkdg_advance(crkdg_ctx* c, int n_steps, double cfl, double t_end, int captu
     const int lim_rest = (c->limiter_on || c->pp_eps > 0.0) ? 1 : 0;
     const double M_first = c->M_pending, M_rest = c->M;
     const double pp_first = c->pp_pending, pp_rest = c->pp_eps;
-    int ns, nseg;
-    strips_segs(c, c->seg_rows, &ns, &nseg);
-    r = ensure_partials(c, (size_t)ns * nseg * 8);
+    r = ensure_step_scratch(c);
     if (r) return r;
     if (use_linear(c)) {   // slots of the modal step too: nothing may allocate while a graph is captured
         r = linear_shape(c);
         if (r) return r;
+        int ns, nseg;
         strips_segs(c, c->lin_seg_rows, &ns, &nseg);
         r = ensure_partials(c, (size_t)ns * nseg * 8);
         if (r) return r;
@@ -768,13 +823,15 @@ static int enqueue_fe(crkdg_ctx* c, const void* in, void* out, double t, double 
     a.s = 1;
     a.tab = c->d_tab_fe;
     int ns, nseg;
-    strips_segs(c, c->seg_rows, &ns, &nseg);
+    step_segs(c, &ns, &nseg);
     a.seg_len = c->seg_rows;
     a.n_strips = ns;
     a.n_segs = nseg;
-    int r = ensure_partials(c, (size_t)ns * nseg * 8);
+    int r = ensure_step_scratch(c);
     if (r) return r;
     a.partials = c->d_partials;
+    a.seam = c->d_seam;
+    a.seams = step_seams(c, nseg, false);
     CK(crk::launch_step2d(c->kphys, c->precision, c->k, c->basis, a, c->wpb, c->stream));
     return CRKDG_OK;
 }

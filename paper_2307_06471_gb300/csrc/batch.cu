@@ -92,9 +92,14 @@ struct crkdg_batch {
     size_t esize, elems;
     std::vector<BatchProblem> probs;
     std::vector<int2> tasks;
+    std::vector<int2> flux, seams;         // the seam launches' blocks: (problem, block)
+    bool use_seams = false;                // (use_seams)
     void* buf[2] = {nullptr, nullptr};
     BatchProblem* d_probs = nullptr;
     int2* d_tasks = nullptr;
+    int2* d_flux = nullptr;
+    int2* d_seams = nullptr;
+    void* d_seam = nullptr;                // seam scratch of all problems
     DevState* d_states = nullptr;
     int* d_curs = nullptr;
     unsigned* d_done = nullptr;
@@ -123,21 +128,43 @@ StepArgs batch_args(const crkdg_batch* b) {
     a.gamma = b->gamma;
     a.seg_len = b->seg_rows;
     a.partials = b->d_partials;
+    a.seam = b->d_seam;
     return a;
 }
 
 // rebuild the task table for the current segment length
 int build_tasks(crkdg_batch* b) {
     b->tasks.clear();
+    b->flux.clear();
+    b->seams.clear();
+    b->use_seams = crk::use_seams(b->esize, b->tab.s, b->nm, false, b->seg_rows, 1);
     int warp0 = 0;
+    long long slots = 0, seam = 0;
+    const size_t room = (size_t)256 << 20;
     for (int p = 0; p < b->n; ++p) {
         BatchProblem& pb = b->probs[p];
+        const size_t values = (size_t)pb.nx * pb.ny * b->nv * b->nm;
+        const size_t seg = crk::seam_values(b->tab.s, b->k + 1, b->nv, b->nm, false,
+                                            b->limit_mode == CRKDG_LIMIT_FUSED, pb.nx);
         pb.n_strips = (pb.nx + 29) / 30;
         pb.n_segs = (pb.ny + b->seg_rows - 1) / b->seg_rows;
+        if (b->use_seams)
+            pb.n_segs = crk::seam_segments(pb.n_segs, seg * b->esize, values * b->esize,
+                                           (size_t)((double)room * values / b->elems));
+        pb.n_seam_blocks = crk::seam_blocks(b->nv, pb.nx, pb.ny, pb.n_segs, 32);
         pb.warp0 = warp0;
+        pb.slot0 = slots;
+        pb.seam0 = seam;
         const int w = pb.n_strips * pb.n_segs;
         for (int i = 0; i < w; ++i) b->tasks.push_back(make_int2(p, i));
+        if (b->use_seams) {
+            const int nf = crk::seam_flux_blocks(b->esize, b->k + 1, pb.nx, pb.n_segs);
+            for (int i = 0; i < nf; ++i) b->flux.push_back(make_int2(p, i));
+            for (int i = 0; i < pb.n_seam_blocks; ++i) b->seams.push_back(make_int2(p, i));
+            seam += (long long)(seg * pb.n_segs);
+        }
         warp0 += w;
+        slots += w + pb.n_seam_blocks;
     }
     // the limiter pass's tiles: 128 cells of one row of one problem
     std::vector<int4> rows;
@@ -145,17 +172,30 @@ int build_tasks(crkdg_batch* b) {
         for (int y = 0; y < b->probs[p].ny; ++y)
             for (int x = 0; x < b->probs[p].nx; x += 128) rows.push_back(make_int4(p, y, x, 0));
     if (b->d_tasks) cudaFree(b->d_tasks);
+    if (b->d_seam) cudaFree(b->d_seam);
+    if (b->d_flux) cudaFree(b->d_flux);
+    if (b->d_seams) cudaFree(b->d_seams);
     if (b->d_partials) cudaFree(b->d_partials);
     if (b->d_rows) cudaFree(b->d_rows);
     b->d_tasks = nullptr;
+    b->d_seam = nullptr;
+    b->d_flux = nullptr;
+    b->d_seams = nullptr;
     b->d_partials = nullptr;
     b->d_rows = nullptr;
     b->n_rows = (int)rows.size();
     BCK(cudaMalloc(&b->d_rows, rows.size() * sizeof(int4)));
     BCK(cudaMemcpy(b->d_rows, rows.data(), rows.size() * sizeof(int4), cudaMemcpyHostToDevice));
     BCK(cudaMalloc(&b->d_tasks, b->tasks.size() * sizeof(int2)));
-    BCK(cudaMalloc(&b->d_partials, std::max((size_t)warp0 * 8, (size_t)b->n * START_BLOCKS) * sizeof(double)));
+    BCK(cudaMalloc(&b->d_partials, std::max((size_t)slots * (b->nv + 2), (size_t)b->n * START_BLOCKS) * sizeof(double)));
     BCK(cudaMemcpy(b->d_tasks, b->tasks.data(), b->tasks.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    if (b->use_seams) {
+        BCK(cudaMalloc(&b->d_flux, b->flux.size() * sizeof(int2)));
+        BCK(cudaMalloc(&b->d_seams, b->seams.size() * sizeof(int2)));
+        BCK(cudaMalloc(&b->d_seam, (size_t)seam * b->esize));
+        BCK(cudaMemcpy(b->d_flux, b->flux.data(), b->flux.size() * sizeof(int2), cudaMemcpyHostToDevice));
+        BCK(cudaMemcpy(b->d_seams, b->seams.data(), b->seams.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    }
     BCK(cudaMemcpy(b->d_probs, b->probs.data(), b->n * sizeof(BatchProblem), cudaMemcpyHostToDevice));
     for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
     b->graphs.clear();
@@ -178,13 +218,11 @@ int enqueue_batch_step(crkdg_batch* b, int limit, double M, double pp) {
         if (e != cudaSuccess) return bfail(CRKDG_ECUDA, std::string("batched limiter pass: ") + cudaGetErrorString(e));
         a.limit = 0;
     }
-    cudaError_t e = b->precision == CRKDG_F32
-                        ? crk::batch2d_euler_f32(b->k, b->basis, a, b->d_probs, b->d_tasks, (int)b->tasks.size(),
-                                                 b->d_states, b->d_curs, b->d_done, b->buf[0], b->buf[1], b->wpb,
-                                                 b->stream)
-                        : crk::batch2d_euler_f64(b->k, b->basis, a, b->d_probs, b->d_tasks, (int)b->tasks.size(),
-                                                 b->d_states, b->d_curs, b->d_done, b->buf[0], b->buf[1], b->wpb,
-                                                 b->stream);
+    a.seams = b->use_seams;
+    const crk::BatchTables t{b->d_probs, b->n, b->d_tasks, b->d_flux, b->d_seams,
+                             (int)b->tasks.size(), (int)b->flux.size(), (int)b->seams.size()};
+    auto step = b->precision == CRKDG_F32 ? crk::batch2d_euler_f32 : crk::batch2d_euler_f64;
+    cudaError_t e = step(b->k, b->basis, a, t, b->d_states, b->d_curs, b->d_done, b->buf[0], b->buf[1], b->wpb, b->stream);
     if (e != cudaSuccess) return bfail(CRKDG_ECUDA, std::string("batched step: ") + cudaGetErrorString(e));
     return CRKDG_OK;
 }
@@ -314,7 +352,7 @@ void crkdg_batch_destroy(crkdg_batch* b) {
     for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
     for (int i = 0; i < 2; ++i)
         if (b->buf[i]) cudaFree(b->buf[i]);
-    for (void* p : {(void*)b->d_probs, (void*)b->d_tasks, (void*)b->d_states, (void*)b->d_curs, (void*)b->d_done,
+    for (void* p : {(void*)b->d_probs, (void*)b->d_tasks, (void*)b->d_flux, (void*)b->d_seams, b->d_seam, (void*)b->d_states, (void*)b->d_curs, (void*)b->d_done,
                     (void*)b->d_partials, (void*)b->d_tab, (void*)b->d_flags, (void*)b->d_rows})
         if (p) cudaFree(p);
     delete b;
@@ -542,10 +580,9 @@ int crkdg_batch_sizes(const crkdg_batch* b, int* n_problems, long long* total_ce
 int crkdg_batch_set_limit_mode(crkdg_batch* b, int mode) {
     if (!b) return bfail(CRKDG_EINVAL, "null batch");
     if (mode != CRKDG_LIMIT_FUSED && mode != CRKDG_LIMIT_PASS) return bfail(CRKDG_EINVAL, "unknown limit mode");
+    if (mode == b->limit_mode) return CRKDG_OK;
     b->limit_mode = mode;
-    for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
-    b->graphs.clear();
-    return CRKDG_OK;
+    return build_tasks(b);   // the seam scratch holds more in the fused mode
 }
 
 int crkdg_batch_set_launch(crkdg_batch* b, int seg_rows, int wpb) {

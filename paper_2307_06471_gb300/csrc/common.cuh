@@ -78,6 +78,8 @@ struct StepArgs {
     int dt_from_dev;
     DevState* ds;
     double* partials;         // per-warp reduction slots
+    int seams;                // the step leaves the faces between segments to the seam launches
+    void* seam;               // seam scratch (step2d.cuh)
     int s;
     const double* tab;        // device tableau buffer, layout of pack_tableau
     BCSide bc[4];             // W, E, S, N
@@ -116,7 +118,10 @@ struct BatchProblem {
     double x0, y0, dx, dy;
     double rx, ry;         // 1/dx, 1/dy (host)
     int n_strips, n_segs;
-    int warp0;             // first task / reduction slot of the problem
+    int warp0;             // first task of the problem
+    int n_seam_blocks;     // blocks of its last seam launch
+    long long slot0;       // its first reduction slot: step warps, then seam blocks
+    long long seam0;       // element offset of its seam scratch
     int sq;                // 1: square cells (dx == dy), the square-cell form of the step
 };
 
@@ -373,6 +378,52 @@ __device__ __forceinline__ void bc_exterior(const BCSide& bc, int axis, const T*
         default:
             break;
     }
+}
+
+// Values per segment of the seam scratch (layout in step2d.cuh): s stages, nq
+// face points, nv variables, nm modes; dev: deviation form; lim: limit on load
+__host__ __device__ inline size_t seam_values(int s, int nq, int nv, int nm, bool dev, bool lim, int nx) {
+    return (size_t)nx * (2 * (s * nq * nv + nq * nv + (dev ? nv : 0)) + nv * nm * (lim ? 2 : 1));
+}
+// The blocks of the last seam launch, at most `most`: a warp per variable and 32
+// cells of the segments' first and last rows (first alone where every segment
+// is one row)
+constexpr int SEAM_CELL_THREADS = 256;
+inline int seam_blocks(int nv, int nx, int ny, int n_segs, int most) {
+    const long long warps = ((long long)nx * n_segs * (n_segs == ny ? 1 : 2) + 31) / 32 * nv;
+    const long long n = (warps + SEAM_CELL_THREADS / 32 - 1) / (SEAM_CELL_THREADS / 32);
+    return (int)(n < most ? n : most);
+}
+// Threads per block and blocks of the flux launch: one warp in FP64, whose pipe
+// one warp fills, so that a small mesh's seams spread over the SMs
+constexpr int SEAM_THREADS_F32 = 128, SEAM_THREADS_F64 = 32;
+inline int seam_flux_blocks(size_t esize, int nq, int nx, int n_segs) {
+    const long long n = (long long)nx * nq * n_segs, t = esize == 4 ? SEAM_THREADS_F32 : SEAM_THREADS_F64;
+    return (int)((n + t - 1) / t);
+}
+// Whether a step whose segments have ny / n_segs rows leaves its seams to the
+// seam launches instead of recomputing the row beyond each end of a segment.
+// FP64 always: its pipe is the bound, and a recomputed row costs what any row
+// does (P^2 SSP-RK3 on 640 x 160, 3 rows a segment: 1.40 ms with halo rows, 0.99
+// with seams; Q^2 RK4 on 80 x 80, 1 row: 0.70 and 0.26 ms).  FP32: the seam
+// launches and their traffic cost about 0.02 ms, so it depends on what a row
+// costs (stages x modes) and on the rows of a segment.  Q^2 RK4 (36) on 1001 x
+// 613, ms per 4 steps with halo rows / seams: 1 row 2.28 / 1.66, 3 rows 1.39 /
+// 1.29, 6 rows 1.17 / 1.13; in the deviation form on 320 x 320, 20 steps, 3
+// rows 1.99 / 1.80, 6 rows 2.92 / 2.60.  P^2 SSP-RK3 (18) on 1920 x 480: 1 row
+// 2.28 / 1.72, 2 rows 1.58 / 1.62, 4 rows 1.23 / 1.29.  P^1 SSP-RK3 (9) on 480 x
+// 120, 2 rows, one step: 0.062 / 0.072.
+inline bool use_seams(size_t esize, int stages, int modes, bool lim_on_load, int ny, int n_segs) {
+    if (esize == 8) return true;
+    const int rows = stages * modes >= 27 ? 6 : (stages * modes >= 18 ? 1 : 0);
+    return !lim_on_load && ny <= (long long)rows * n_segs;
+}
+// Segments that keep the seam scratch within an eighth of a state copy (or
+// 256 MiB): a launch shape asks for memory in proportion to its segments
+inline int seam_segments(int n_segs, size_t seg_bytes, size_t state_bytes, size_t room = (size_t)256 << 20) {
+    const size_t cap = state_bytes / 8 > room ? state_bytes / 8 : room;
+    const size_t most = cap / (seg_bytes ? seg_bytes : 1);
+    return (size_t)n_segs <= most ? n_segs : (most ? (int)most : 1);
 }
 
 // Affine forms of the boundary sides (see BCSide); the kernels fall back to

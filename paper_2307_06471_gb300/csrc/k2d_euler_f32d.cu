@@ -9,10 +9,10 @@
 namespace crk {
 namespace {
 
-template <int K, int B, bool SQ>
+template <int K, int B, bool SQ, bool SEAM>
 cudaError_t run_step_dt(const StepArgs& a, int wpb, cudaStream_t st) {
     using C = Step2D<float, K, B, PHYS_EULER>;
-    auto kern = step2d_kernel<float, K, B, PHYS_EULER, true, false, false, true, SQ>;
+    auto kern = step2d_kernel<float, K, B, PHYS_EULER, true, false, false, true, SQ, SEAM>;
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
@@ -27,17 +27,17 @@ cudaError_t run_step_dt(const StepArgs& a, int wpb, cudaStream_t st) {
     kern<<<(total + wpb - 1) / wpb, threads, smem, st>>>(b);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_finalize<4>(b, st);
+    if constexpr (SEAM) return launch_seam<float, K, B, PHYS_EULER, true, true, SQ>(b, st);
+    else return launch_finalize<4>(b, st);
 }
 
 // square cells (dx == dy) take the square-cell form for k = 2
 template <int K, int B>
 cudaError_t run_step_d(const StepArgs& a, int wpb, cudaStream_t st) {
-#ifndef CRK_SQ_STEP_OFF
     if constexpr (K == 2)
-        if (a.dx == a.dy) return run_step_dt<K, B, true>(a, wpb, st);
-#endif
-    return run_step_dt<K, B, false>(a, wpb, st);
+        if (a.dx == a.dy)
+            return a.seams ? run_step_dt<K, B, true, true>(a, wpb, st) : run_step_dt<K, B, true, false>(a, wpb, st);
+    return a.seams ? run_step_dt<K, B, false, true>(a, wpb, st) : run_step_dt<K, B, false, false>(a, wpb, st);
 }
 
 template <int K, int B>

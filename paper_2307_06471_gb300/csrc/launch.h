@@ -90,11 +90,18 @@ cudaError_t info_step2d_linear(int prec, int k, int basis, int s, KernelInfo* in
 cudaError_t launch_f64_to_f32(const double* in, float* out, size_t n, int comp, cudaStream_t st);
 cudaError_t launch_f32_to_f64(const float* in, double* out, size_t n, int comp, cudaStream_t st);
 
-struct BatchProblem;
+// the tables of a batched step's launches
+struct BatchTables {
+    const BatchProblem* probs;
+    int n_probs;
+    const int2 *tasks, *flux, *seams;
+    int n_tasks, n_flux, n_seams;
+};
+
 #define CRK_DECL_B(NAME)                                                                                     \
-    cudaError_t batch2d_##NAME(int k, int basis, const StepArgs& a, const BatchProblem* probs, const int2* tasks, \
-                               int n_tasks, DevState* states, int* curs, unsigned* done, const void* bufA,    \
-                               void* bufB, int wpb, cudaStream_t st);                                         \
+    cudaError_t batch2d_##NAME(int k, int basis, const StepArgs& a, const BatchTables& t, DevState* states,      \
+                               int* curs, unsigned* done, const void* bufA, void* bufB, int wpb,              \
+                               cudaStream_t st);                                                              \
     cudaError_t binfo2d_##NAME(int k, int basis, int s, KernelInfo* info);                                 \
     cudaError_t blimit2d_##NAME(int k, int basis, const StepArgs& a, const BatchProblem* probs, const int4* rows, \
                                 int n_rows, DevState* states, const int* curs, void* bufA, void* bufB,        \

@@ -15,30 +15,30 @@
 //      kept per stage in the same thread's shared-memory slot;
 //   4. completes the update of the row below (its north face is the current
 //      row's south face) and writes u^{n+1} of that row once.
-// Halo columns and one extra row at each segment end are recomputed instead
-// of exchanged: the compactness of cRKDG (Sec. 3.1) means one ring suffices.
+// Halo columns are recomputed instead of exchanged: the compactness of cRKDG
+// (Sec. 3.1) means one ring suffices.  So is the row beyond each end of a
+// segment, two rows per segment, where rows are cheap or segments long (2 of 28
+// rows on the 1920 x 480 mesh).  Elsewhere (use_seams) the faces between two
+// segments (seams) are left to two small launches: a segment keeps its first
+// row's south and its last row's north traces in a scratch array and the two
+// rows' updates unfinished; seam_flux_kernel forms the seams' fluxes, seam_kernel
+// completes the rows and ends the step.  Both ways do the same operations in the
+// same order for every cell: the result does not depend on the segments, bit for
+// bit.  (Completing a seam at the end of the warp that finished last, by a
+// counter per row, was slower than the launches: 2.48 against 2.26 ms for two
+// steps of P^2 in FP64 on 640 x 160, 2.45 against 1.82 ms for twenty of the
+// deviation form on 320 x 320: each warp's end was a chain of fences, atomics and
+// loads.)
 // Boundary data enter only the final-stage fluxes, at t^n + c_i dt (Sec. 3.4).
 // The FP64 epilogue reduces the new cell averages (max wave speed, totals;
-// eq. (3.4)) per warp; finalize_step_kernel (a batch: the problem's last warp)
-// combines the warps' slots and updates the device run state.
+// eq. (3.4)) per warp; the launch that ends the step (finalize_step_kernel or
+// seam_kernel) combines the warps' slots and updates the device run state.
 #pragma once
 #include "common.cuh"
+#include "launch.h"
 #include "limiter.cuh"
 #include "mlp_warp.cuh"
 
-// where the per-row accumulator sum_i b_i vol_i lives: 0 registers, 1 the
-// thread's shared-memory slot (tuning knob)
-#ifndef CRK_V_SMEM
-#define CRK_V_SMEM 0
-#endif
-// 1: stages with a local operator form the east/south Lax--Friedrichs fluxes
-// from the physical fluxes that operator already computed (own traces), the
-// neighbouring lane's (shuffle) and the row below's (kept in shared memory).
-// Off: measured slower (fewer instructions, more shuffle and shared-memory
-// latency in the inner loop: 0.269 against 0.260 ms per step kernel)
-#ifndef CRK_LF_REUSE
-#define CRK_LF_REUSE 0
-#endif
 // launch bounds of the single-problem step kernel (tuning knobs)
 #ifndef CRK_STEP_MAXT
 #define CRK_STEP_MAXT 256
@@ -115,13 +115,49 @@ struct Step2D {
     static constexpr int NRED = NV + 2;   // reduction slots: maxspeed, sums[NV], troubled
 
     // T elements of private shared memory per thread for s stages: L_j
-    // (j < s-1), north traces per stage, pending update, (CRK_V_SMEM) the
-    // row's sum_i b_i vol_i, and (CRK_LF_REUSE) the north traces' normal
-    // fluxes and wave speeds per stage
-    static __host__ __device__ constexpr int smem_per_thread(int s) {
-        return (s - 1) * NDOF + s * NQ * NV + NDOF + (CRK_V_SMEM ? NDOF : 0) + (CRK_LF_REUSE ? s * NQ * (NV + 1) : 0);
+    // (j < s-1), north traces per stage, pending update
+    static __host__ __device__ constexpr int smem_per_thread(int s) { return (s - 1) * NDOF + s * NQ * NV + NDOF; }
+};
+
+// The seam scratch of the segments, per segment and column: the first row's
+// south traces (per stage), the last row's north traces, the first row's
+// north-face flux (and, in deviation form, its move between the two rows' bases),
+// the flux of the seam below it (likewise), its volume term and, with the limit
+// on load, its limited u^n.  Values of
+// entry k of all columns lie together.  (Its east/west face terms wait in the
+// output buffer, as a last row's update does.)
+template <class T, int K, int B, int PHYS, bool DEV>
+struct Seam {
+    using C = Step2D<T, K, B, PHYS>;
+    static constexpr int NF = C::NQ * C::NV;
+    T* base;
+    size_t nx, seg_size;
+    int ntr;
+    __device__ __forceinline__ Seam(void* scratch, int s, int nx_, bool lim)
+        : base(static_cast<T*>(scratch)), nx(nx_), seg_size(seam_values(s, C::NQ, C::NV, C::NM, DEV, lim, nx_)),
+          ntr(s * NF) {}
+    __device__ __forceinline__ T* at(int seg, int k, int col) const { return base + seg * seg_size + k * nx + col; }
+    __device__ __forceinline__ T* south(int seg, int k, int col) const { return at(seg, k, col); }
+    __device__ __forceinline__ T* north(int seg, int k, int col) const { return at(seg, ntr + k, col); }
+    __device__ __forceinline__ T* flux(int seg, int k, int col) const { return at(seg, 2 * ntr + k, col); }
+    // the flux of the seam below the segment (and its move between bases)
+    __device__ __forceinline__ T* below(int seg, int k, int col) const {
+        return at(seg, 2 * ntr + NF + (DEV ? C::NV : 0) + k, col);
+    }
+    __device__ __forceinline__ T* vol(int seg, int k, int col) const {
+        return at(seg, 2 * (ntr + NF + (DEV ? C::NV : 0)) + k, col);
+    }
+    __device__ __forceinline__ T* un(int seg, int k, int col) const {
+        return at(seg, 2 * (ntr + NF + (DEV ? C::NV : 0)) + C::NDOF + k, col);
     }
 };
+
+// First row of segment seg of nseg (rows split evenly); the 64-bit division
+// only where the product needs it
+__device__ __forceinline__ int seg_row(int seg, int ny, int nseg) {
+    const unsigned long long n = (unsigned long long)seg * ny;
+    return n >> 32 ? (int)(n / nseg) : (int)((unsigned)n / (unsigned)nseg);
+}
 
 // Per-problem view of one step.  The single-problem kernel reads the mesh
 // straight from its launch arguments (kernel-parameter constant bank, no
@@ -145,11 +181,11 @@ struct ArgsView {
     __device__ __forceinline__ int seg_len() const { return a.seg_len; }
     __device__ __forceinline__ int total_warps() const { return a.n_strips * a.n_segs; }
     __device__ __forceinline__ double* partials() const { return a.partials; }
+    __device__ __forceinline__ void* seam() const { return a.seam; }
     __device__ __forceinline__ DevState* ds() const { return a.ds; }
     __device__ __forceinline__ int* cur() const { return nullptr; }
     __device__ __forceinline__ unsigned* done() const { return nullptr; }
     __device__ __forceinline__ bool copy_if_idle() const { return true; }
-    static constexpr bool kLastWarp = false;   // finalize_step_kernel ends the step
     // derived constants, computed on the host (set_derived)
     __device__ __forceinline__ T rxT() const {
         if constexpr (sizeof(T) == 4) return a.rxf;
@@ -179,9 +215,10 @@ struct ProbView {
     double x0_, y0_, dx_, dy_;
     double t_, dt_;
     int n_strips_, n_segs_, seg_len_, total_warps_;
-    double* partials_;    // this problem's per-warp reduction slots
+    double* partials_;    // this problem's reduction slots
+    void* seam_;          // this problem's seam scratch
     DevState* ds_;        // this problem's run state
-    int* cur_;            // this problem's buffer index (flipped by its last warp)
+    int* cur_;            // this problem's buffer index (flipped at the end of its step)
     unsigned* done_;      // count of problems that reached t_end
     __device__ __forceinline__ const T* uin() const { return uin_; }
     __device__ __forceinline__ T* uout() const { return uout_; }
@@ -198,11 +235,11 @@ struct ProbView {
     __device__ __forceinline__ int seg_len() const { return seg_len_; }
     __device__ __forceinline__ int total_warps() const { return total_warps_; }
     __device__ __forceinline__ double* partials() const { return partials_; }
+    __device__ __forceinline__ void* seam() const { return seam_; }
     __device__ __forceinline__ DevState* ds() const { return ds_; }
     __device__ __forceinline__ int* cur() const { return cur_; }
     __device__ __forceinline__ unsigned* done() const { return done_; }
     __device__ __forceinline__ bool copy_if_idle() const { return false; }
-    static constexpr bool kLastWarp = true;    // the problem's last warp ends its step
     // per-problem constants, in the arithmetic of set_derived (1/dx and 1/dy
     // from the problem table, made on the host)
     double rx_, ry_, M_, bx_, by_;
@@ -219,7 +256,8 @@ struct ProbView {
 // cfl, t_end, lim_count: the run state's values (not written by the step)
 __device__ __forceinline__ void finish_run_state(const StepArgs& a, DevState* ds, double mx, const double* sm_,
                                                  int nv, double tr, double t0, double dt, double cfl,
-                                                 double t_end, unsigned lim_count, int* cur, unsigned* done) {
+                                                 double t_end, unsigned long long lim_count, int* cur,
+                                                 unsigned* done) {
     ds->maxspeed = mx;
     for (int v = 0; v < nv; ++v) ds->sums[v] = sm_[v];
     // troubled cells: this step's limit-on-load, else a separate pass over u^n
@@ -239,162 +277,122 @@ __device__ __forceinline__ void finish_run_state(const StepArgs& a, DevState* ds
     if (done && reached) atomicAdd(done, 1u);
 }
 
+// NV values summed over a warp's lanes (every lane returns lane v's sum of
+// value v, v < NV): the lanes of a pair each take over half of the values, so
+// four FP64 sums need 6 additions a lane instead of 20 (FP64 runs at 1/64 of
+// the FP32 rate).
+template <int NV>
+__device__ __forceinline__ void warp_sums(double (&v)[NV]) {
+    const int lane = threadIdx.x & 31;
+    constexpr unsigned ALL = 0xffffffffu;
+    if constexpr (NV == 4) {
+        const bool h = lane & 16, q = lane & 8;
+        const double a0 = (h ? v[2] : v[0]) + __shfl_xor_sync(ALL, h ? v[0] : v[2], 16);
+        const double a1 = (h ? v[3] : v[1]) + __shfl_xor_sync(ALL, h ? v[1] : v[3], 16);
+        double x = (q ? a1 : a0) + __shfl_xor_sync(ALL, q ? a0 : a1, 8);
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) x += __shfl_xor_sync(ALL, x, off);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = __shfl_sync(ALL, x, 8 * i);
+    } else {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+            for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(ALL, v[i], off);
+    }
+}
+
 // FP64 epilogue of a step: warp reduction of the lane accumulators (max
 // wave speed, NV totals, troubled count, status bits) into the warp's slot
-// (NV + 2 doubles).  Single problems (PV::kLastWarp false) leave the rest to
-// finalize_step_kernel, launched after the step; in a batch the last warp of
-// a problem to arrive (atomic counter, no waiting) reduces that problem's
-// slots in a fixed order and updates its run state.
+// (NV + 2 doubles; the totals without the cell's area, the maximum as an
+// ordered key, the count as an integer, both stored bitwise).  The launch that
+// follows the step reduces the slots.
 template <int NV, int NRED, class PV>
-__device__ __forceinline__ void step_epilogue(const StepArgs& a, const PV& pv, int gw, int lane, int total_warps,
-                                              double red_max, double* red_sum, unsigned red_trouble,
-                                              unsigned status, double cell, double t0, double dt) {
+__device__ __forceinline__ void step_epilogue(const PV& pv, int gw, int lane, double red_max, double (&red_sum)[NV],
+                                              unsigned red_trouble, unsigned status) {
     static_assert(NRED == NV + 2, "slot layout: max speed, NV totals, troubled count");
+    unsigned long long key = speed_key(red_max);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        red_max = fmax(red_max, __shfl_xor_sync(0xffffffffu, red_max, off));
-#pragma unroll
-        for (int v = 0; v < NV; ++v) red_sum[v] += __shfl_xor_sync(0xffffffffu, red_sum[v], off);
-        red_trouble += __shfl_xor_sync(0xffffffffu, red_trouble, off);
-        status |= __shfl_xor_sync(0xffffffffu, status, off);
+        const unsigned long long k = __shfl_xor_sync(0xffffffffu, key, off);
+        key = k > key ? k : key;
     }
-    double* slotp = pv.partials() + (size_t)gw * NRED;
-    unsigned prev = 0;
+    warp_sums<NV>(red_sum);
+    red_trouble = __reduce_add_sync(0xffffffffu, red_trouble);
+    status = __reduce_or_sync(0xffffffffu, status);
     if (lane == 0) {
-        slotp[0] = red_max;
+        double* slotp = pv.partials() + (size_t)gw * NRED;
+        slotp[0] = __longlong_as_double((long long)key);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) slotp[1 + v] = red_sum[v] * cell;
-        slotp[1 + NV] = __longlong_as_double((long long)red_trouble);   // an integer, stored bitwise
+        for (int v = 0; v < NV; ++v) slotp[1 + v] = red_sum[v];
+        slotp[1 + NV] = __longlong_as_double((long long)red_trouble);
         if (status) atomicOr(&pv.ds()->status, status);
-        if constexpr (PV::kLastWarp) {
-            __threadfence();
-            prev = atomicAdd(&pv.ds()->counter, 1u);
-        }
-    }
-    if constexpr (!PV::kLastWarp) {
-        return;
-    } else {
-        prev = __shfl_sync(0xffffffffu, prev, 0);
-        if (prev != (unsigned)total_warps - 1) return;
-        // last warp: fixed-order reduction of all per-warp slots (deterministic)
-        __threadfence();
-        double mx = 0.0, sm_[NV], tr = 0.0;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) sm_[v] = 0.0;
-        for (int wi = lane; wi < total_warps; wi += 32) {
-            const double* q = pv.partials() + (size_t)wi * NRED;
-            mx = fmax(mx, __ldcg(q));
-#pragma unroll
-            for (int v = 0; v < NV; ++v) sm_[v] += __ldcg(q + 1 + v);
-            tr += double(__double_as_longlong(__ldcg(q + 1 + NV)));
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-#pragma unroll
-            for (int v = 0; v < NV; ++v) sm_[v] += __shfl_xor_sync(0xffffffffu, sm_[v], off);
-            tr += __shfl_xor_sync(0xffffffffu, tr, off);
-        }
-        if (lane == 0) {
-            DevState* ds = pv.ds();
-            finish_run_state(a, ds, mx, sm_, NV, tr, t0, dt, ds->cfl, ds->t_end, ds->lim_count, pv.cur(), pv.done());
-        }
     }
 }
 
-// The end of a single-problem step, as its own launch of one block (the
-// step's slots are complete when it starts): each thread reduces a run of
-// slots with their loads in flight together, then fixed-order trees
-// (deterministic); thread 0 updates the device run state.  A last warp of the
-// step itself would reduce ~1,000-2,400 slots alone while the rest of the GPU
-// idles.  The block runs on one SM, whose FP64 pipe (1/64 of the FP32 rate)
-// would bound it: only the NV totals are added in FP64; the maximum wave
-// speed is taken on the bit patterns (non-negative doubles order as integers)
-// and the troubled count is an integer.
-constexpr int FINALIZE_THREADS = 256;
-
+// What a block holds of the reductions, and the sum over its threads (fixed
+// order: deterministic); thread 0 holds the result.
 template <int NV>
-__global__ void __launch_bounds__(FINALIZE_THREADS) finalize_step_kernel(const StepArgs a, int total_warps) {
-    constexpr int NRED = NV + 2;
-    // launched as a programmatic dependent of the step: wait here until the
-    // step grid has completed and its writes are visible
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    DevState* ds = a.ds;
-    // every load is issued before any result is needed: the run state (none
-    // of these fields is written by the step) and the thread's slots
-    const double t0 = a.dt_from_dev ? ds->t : a.t;
-    const double dt = a.dt_from_dev ? ds->dt : a.dt;
-    const double cfl = ds->cfl, t_end = ds->t_end;
-    const unsigned lim_count = ds->lim_count;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    unsigned long long mk = 0, tr = 0;
-    double sm_[NV];
+struct StepRed {
+    unsigned long long key = 0, trouble = 0;
+    double sum[NV] = {};
+    __device__ __forceinline__ void add_slot(const double* q) {
+        double e[NV + 2];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sm_[v] = 0.0;
-    // chunks of PER slots per thread, loaded unconditionally from valid
-    // addresses (slot 0 past the end, masked) so that all are in flight at once
-    constexpr int PER = 8;
-    for (int base = threadIdx.x; base < total_warps; base += PER * FINALIZE_THREADS) {
-        double qv[PER][NRED];
+        for (int i = 0; i < NV + 2; ++i) e[i] = __ldcg(q + i);
+        const unsigned long long k = (unsigned long long)__double_as_longlong(e[0]);
+        key = k > key ? k : key;
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int wi = base + k * FINALIZE_THREADS;
-            const double* q = a.partials + (size_t)(wi < total_warps ? wi : 0) * NRED;
-#pragma unroll
-            for (int e = 0; e < NRED; ++e) qv[k][e] = q[e];
-        }
-#pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            if (base + k * FINALIZE_THREADS >= total_warps) break;
-            const unsigned long long key = speed_key(qv[k][0]);
-            mk = key > mk ? key : mk;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) sm_[v] += qv[k][1 + v];
-            tr += (unsigned long long)__double_as_longlong(qv[k][1 + NV]);
-        }
+        for (int v = 0; v < NV; ++v) sum[v] += e[1 + v];
+        trouble += (unsigned long long)__double_as_longlong(e[1 + NV]);
     }
-    auto warp_tree = [&]() {
+    __device__ __forceinline__ void put_slot(double* q) const {
+        q[0] = __longlong_as_double((long long)key);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) q[1 + v] = sum[v];
+        q[1 + NV] = __longlong_as_double((long long)trouble);
+    }
+    __device__ __forceinline__ void warp_reduce() {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long k = __shfl_xor_sync(0xffffffffu, mk, off);
-            mk = k > mk ? k : mk;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) sm_[v] += __shfl_xor_sync(0xffffffffu, sm_[v], off);
-            tr += __shfl_xor_sync(0xffffffffu, tr, off);
+            const unsigned long long k = __shfl_xor_sync(0xffffffffu, key, off);
+            key = k > key ? k : key;
+            trouble += __shfl_xor_sync(0xffffffffu, trouble, off);
         }
-    };
-    if (!(dt > 0.0)) return;   // the step left the state and the run state unchanged
-    warp_tree();
-    constexpr int NW = FINALIZE_THREADS / 32;
-    __shared__ unsigned long long red_k[NW], red_t[NW];
-    __shared__ double red_s[NW][NV];
-    if (lane == 0) {
-        red_k[w] = mk;
-        red_t[w] = tr;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) red_s[w][v] = sm_[v];
+        warp_sums<NV>(sum);
     }
-    __syncthreads();
-    if (w != 0) return;
-    mk = lane < NW ? red_k[lane] : 0ull;
-    tr = lane < NW ? red_t[lane] : 0ull;
+    template <int NT>
+    __device__ __forceinline__ void block_reduce() {
+        warp_reduce();
+        if constexpr (NT > 32) {
+            constexpr int NW = NT / 32;
+            __shared__ double slots[NW][NV + 2];
+            const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+            __syncthreads();   // an earlier call's slots have been read
+            if (lane == 0) put_slot(slots[w]);
+            __syncthreads();
+            if (threadIdx.x == 0)
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sm_[v] = lane < NW ? red_s[lane][v] : 0.0;
-    warp_tree();
-    if (lane == 0)
-        finish_run_state(a, ds, __longlong_as_double((long long)mk), sm_, NV, double(tr), t0, dt, cfl, t_end, lim_count,
-                         nullptr, nullptr);
-}
+                for (int i = 1; i < NW; ++i) {
+                    const unsigned long long k = (unsigned long long)__double_as_longlong(slots[i][0]);
+                    key = k > key ? k : key;
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) sum[v] += slots[i][1 + v];
+                    trouble += (unsigned long long)__double_as_longlong(slots[i][1 + NV]);
+                }
+        }
+    }
+};
 
-// launch of finalize_step_kernel after a single-problem step launched with b,
-// as a programmatic dependent launch: the step's blocks allow it early
-// (griddepcontrol.launch_dependents), so its block is scheduled as soon as an
-// SM has room and only waits for the step's completion, without a launch gap
-template <int NV>
-inline cudaError_t launch_finalize(const StepArgs& b, cudaStream_t st) {
+// A step kernel's follow-up launch as its programmatic dependent: the step's
+// blocks allow it early (griddepcontrol.launch_dependents), so its blocks are
+// scheduled as soon as an SM has room and wait for the step's completion,
+// without a launch gap
+template <class... A, class... V>
+inline cudaError_t launch_dependent(void (*kern)(A...), int grid, int threads, cudaStream_t st, V... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3(FINALIZE_THREADS);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -402,11 +400,189 @@ inline cudaError_t launch_finalize(const StepArgs& b, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, finalize_step_kernel<NV>, b, b.n_strips * b.n_segs);
+    return cudaLaunchKernelEx(&cfg, kern, A(args)...);
+}
+// ... which waits here until the step grid has completed and its writes are visible
+__device__ __forceinline__ void wait_for_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The end of a single-problem step without seams, as its own launch of one block: each
+// thread reduces a run of slots, then fixed-order trees; thread 0 updates the
+// device run state.  A last warp of the step itself would reduce ~1,000-2,400
+// slots alone while the rest of the GPU idles.
+constexpr int FINALIZE_THREADS = 256;
+
+template <int NV>
+__global__ void __launch_bounds__(FINALIZE_THREADS) finalize_step_kernel(const StepArgs a, int total_warps) {
+    wait_for_step();
+    DevState* ds = a.ds;
+    const double dt = a.dt_from_dev ? ds->dt : a.dt;
+    if (!(dt > 0.0)) return;   // the step left the state and the run state unchanged
+    StepRed<NV> red;
+#pragma unroll 4
+    for (int w = threadIdx.x; w < total_warps; w += FINALIZE_THREADS)
+        red.add_slot(a.partials + (size_t)w * (NV + 2));
+    red.template block_reduce<FINALIZE_THREADS>();
+    if (threadIdx.x == 0) {
+        for (int v = 0; v < NV; ++v) red.sum[v] *= a.cell;
+        finish_run_state(a, ds, __longlong_as_double((long long)red.key), red.sum, NV, double(red.trouble),
+                         a.dt_from_dev ? ds->t : a.t, dt, ds->cfl, ds->t_end, ds->lim_count, nullptr, nullptr);
+    }
+}
+
+template <int NV>
+inline cudaError_t launch_finalize(const StepArgs& b, cudaStream_t st) {
+    return launch_dependent(&finalize_step_kernel<NV>, 1, FINALIZE_THREADS, st, b, b.n_strips * b.n_segs);
 }
 
 // In a step kernel: its dependent finalize launch may be scheduled now
 __device__ __forceinline__ void allow_dependent_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+// The accumulators of the new averages' reductions: FP32 states (plain or
+// compensated) keep the maximum in FP32 (GB300's FP64 pipe is 1/64 of its FP32
+// rate) and the totals in compensated FP32 (TwoSum; a compensated state adds
+// its lo parts into the error term), converted to FP64 once per warp; FP64
+// states keep FP64.
+template <class T, int NV>
+struct CellRed {
+    T hi[NV] = {}, lo[NV] = {};   // FP32: totals and their error terms
+    T maxT = T(0);
+    double max = 0.0;
+    double sum[NV] = {};          // FP64
+    unsigned status = 0;
+    // FP64 maximum and totals (adv_speed: the one speed of a linear flux, 0 where no cell was written)
+    template <int PHYS>
+    __device__ __forceinline__ void close(double adv_speed) {
+        if constexpr (sizeof(T) == 4) {
+            max = PHYS == PHYS_EULER ? double(maxT) : adv_speed;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) sum[v] = double(hi[v]) + double(lo[v]);
+        }
+    }
+};
+
+// Wave speed of new averages A, in the state's arithmetic, and its status bits
+template <class T, int PHYS, int NV, class PV>
+__device__ __forceinline__ T new_speed(const StepArgs& a, const PV& pv, const T* A, T rx, T ry, T gm1, T gam,
+                                       unsigned& status) {
+    if constexpr (PHYS != PHYS_EULER) {
+        if (!(A[0] == A[0])) status |= ST_NAN;
+        return T(pv.adv_speed());
+    } else {
+        const T ir = T(1) / A[0];
+        const T w = A[1] * ir, vv = A[2] * ir;
+        const T p = gm1 * (A[3] - T(0.5) * (A[1] * w + A[2] * vv));
+        const T c = sqrt(fmax(gam * p * ir, T(0)));
+        T sp;
+        if constexpr (sizeof(T) == 4) sp = (fabs(w) + c) * rx + (fabs(vv) + c) * ry;
+        else sp = (fabs(w) + c) / pv.dx() + (fabs(vv) + c) / pv.dy();
+        if (!(A[0] > T(0)) || !(p > T(0))) status |= ST_NONPHYSICAL;
+        if (!(sp == sp)) status |= ST_NAN;
+        return sp;
+    }
+}
+
+// hi' + lo' = hi + lo + inc at element ix of a compensated state (TwoSum)
+template <class T>
+__device__ __forceinline__ void store_comp(const T* __restrict__ uin, T* __restrict__ uout, size_t ix, size_t lo_off,
+                                           T inc, T& hi_out, T& lo_out) {
+    const T hi = uin[ix], lo = uin[lo_off + ix];
+    const T d = inc + lo;
+    const T sum = hi + d;
+    const T bv = sum - hi;
+    const T err = (hi - (sum - bv)) + (d - bv);
+    uout[ix] = sum;
+    uout[lo_off + ix] = err;
+    hi_out = sum;
+    lo_out = err;
+}
+
+// u^{n+1} of a cell from its finished update P (COMP: the increment, added to
+// hi + lo; P[v][0] becomes the new hi average) and its part of the reductions
+template <class T, int PHYS, int NV, int NM, bool COMP, class PV>
+__device__ __forceinline__ void store_cell(const StepArgs& a, const PV& pv, const T* __restrict__ uin,
+                                           T* __restrict__ uout, size_t plane, size_t o, T (&P)[NV][NM], T rx, T ry,
+                                           T gm1, T gam, CellRed<T, NV>& red) {
+    static_assert(!COMP || sizeof(T) == 4, "the compensated state is FP32");
+    T avl[NV], A[NV];   // COMP: lo parts of the new averages
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const size_t ix = (size_t)(v * NM + m) * plane + o;
+            if constexpr (COMP) {
+                T hi, lo;
+                store_comp(uin, uout, ix, (size_t)(NV * NM) * plane, P[v][m], hi, lo);
+                if (m == 0) {
+                    P[v][0] = hi;
+                    avl[v] = lo;
+                }
+            } else {
+                uout[ix] = P[v][m];
+            }
+        }
+        A[v] = P[v][0];
+    }
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {   // TwoSum: hi + lo += A[v] exactly
+            const T x = A[v];
+            const T sum = red.hi[v] + x;
+            const T bv = sum - red.hi[v];
+            red.lo[v] += (red.hi[v] - (sum - bv)) + (x - bv);
+            if constexpr (COMP) red.lo[v] += avl[v];
+            red.hi[v] = sum;
+        }
+        const T sp = new_speed<T, PHYS, NV>(a, pv, A, rx, ry, gm1, gam, red.status);
+        if constexpr (PHYS == PHYS_EULER) red.maxT = fmax(red.maxT, sp);
+    } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) red.sum[v] += A[v];
+        red.max = fmax(red.max, new_speed<T, PHYS, NV>(a, pv, A, rx, ry, gm1, gam, red.status));
+    }
+}
+
+// One variable's update of a row in two parts, the same operations wherever a
+// row is completed.  First: sx the east/west face terms, V the volume term, FS the
+// flux of the south face; P = u^n (COMP: 0) minus dt times the operator without
+// its north face.
+template <class T, int K, int B, bool COMP, bool SQ, int NQ, int NM>
+__device__ __forceinline__ void row_update(T (&P)[NM], const T (&sx)[NM], const T (&V)[NM], const T (&FS)[NQ],
+                                           const T (&un)[NM], T rx, T ry, T tdt) {
+    constexpr Tab2D<K, B> tb = make_tab2d<K, B>();
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+        T sy = T(0);
+#pragma unroll
+        for (int p = 0; p < NQ; ++p)
+            if (tb.pS[p][m] != 0.0) sy = fma(FS[p], T(-tb.pS[p][m]), sy);
+        const T fsum = SQ ? fma(rx, sx[m] + sy, -V[m]) : fma(rx, sx[m], ry * sy) - V[m];
+        const T tc = tdt * T(tb.cm[m]);
+        if constexpr (COMP) P[m] = -tc * fsum;
+        else P[m] = fma(-tc, fsum, un[m]);
+    }
+}
+// ... and the north face: FN its flux (DEV: relative to the base of the row
+// above, gS moves it to this row's)
+template <class T, int K, int B, bool DEV, int NQ, int NM>
+__device__ __forceinline__ void add_north(T (&P)[NM], const T (&FN)[NQ], T gS, T ry, T tdt) {
+    constexpr Tab2D<K, B> tb = make_tab2d<K, B>();
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+        T s = T(0);
+#pragma unroll
+        for (int p = 0; p < NQ; ++p)
+            if (tb.pN[p][m] != 0.0) s = fma(FN[p], T(tb.pN[p][m]), s);
+        if constexpr (DEV) {
+            if (tb.sN[m] != 0.0) s = fma(gS, T(-tb.sN[m]), s);
+        }
+        P[m] = fma(-(tdt * T(tb.cm[m])), ry * s, P[m]);
+    }
+}
+template <int NQ, int NV, class T>
+__device__ __forceinline__ void column(const T (&F)[NQ][NV], int v, T (&out)[NQ]) {
+#pragma unroll
+    for (int p = 0; p < NQ; ++p) out[p] = F[p][v];
+}
 
 // COMP = true: compensated FP32 state.  The buffers hold hi planes followed
 // by lo planes (u = hi + lo); every stage computes in T from hi, and only the
@@ -441,12 +617,12 @@ constexpr size_t mlp_smem_bytes(int nthr) {
 // accumulate without the 1/dx factors, applied once to each local-operator
 // value and to the update (rx (sx + sy) - V for rx sx + ry sy - V): 4 packed
 // multiplications per face point fewer.
-template <class T, int K, int B, int PHYS, bool COMP = false, bool MLPI = false, bool LIM = true, bool DEV = false,
-          bool SQ = false, class PV>
+// SEAM = true: the faces between segments are left to the seam launches;
+// false: the row beyond each end of the segment is recomputed instead.
+template <class T, int K, int B, int PHYS, bool COMP, bool MLPI, bool LIM, bool DEV, bool SQ, bool SEAM, class PV>
 __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, const int gw) {
-    static_assert(!DEV || (COMP && PHYS == PHYS_EULER && sizeof(T) == 4 && !MLPI && !LIM && !CRK_LF_REUSE),
+    static_assert(!DEV || (COMP && PHYS == PHYS_EULER && sizeof(T) == 4 && !MLPI && !LIM),
                   "the deviation form is built for the compensated FP32 2D Euler step without limiters");
-    static_assert(!SQ || !CRK_LF_REUSE, "the square-cell form is built without the reused face fluxes");
     using C = Step2D<T, K, B, PHYS>;
     using TBL = typename C::TB;
     constexpr int NQ = C::NQ, NQV = C::NQV, NM = C::NM, NV = C::NV;
@@ -459,8 +635,6 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
     const int S = a.s;
     const int offN = (S - 1) * C::NDOF;
     const int offP = offN + S * NQ * NV;
-    const int offV = offP + C::NDOF;
-    const int offNF = offV + (CRK_V_SMEM ? C::NDOF : 0);   // north fluxes + speeds (CRK_LF_REUSE)
     // the thread's private slots: its warp holds smem_per_thread(S) rows of
     // 32 values, one column per lane (consecutive lanes in consecutive banks),
     // so that slot k sits k * 32 values past the thread's own base
@@ -468,8 +642,6 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
     auto slot = [&](int k) -> T& { return smt[k * 32]; };
 
     const int lane = tid & 31;
-    const int total_warps = pv.total_warps();
-
     const int nx = pv.nx(), ny = pv.ny();
     const size_t plane = (size_t)nx * ny;
     const T* __restrict__ uin = pv.uin();
@@ -491,10 +663,12 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
     const bool has_bcE = !perx && xs + 30 >= nx;
 
     // rows split evenly over the segments (each at most seg_len rows)
-    const int r0 = (int)(((long long)seg * ny) / pv.n_segs());
-    const int r1 = (int)(((long long)(seg + 1) * ny) / pv.n_segs());
-    const int rstart = (r0 > 0 || pery) ? r0 - 1 : r0;
-    const int rend = (r1 < ny || pery) ? r1 : r1 - 1;
+    const int r0 = seg_row(seg, ny, pv.n_segs()), r1 = seg_row(seg + 1, ny, pv.n_segs());
+    // the faces below the first and above the last row that are seams, or the
+    // halo rows that are recomputed for them
+    const bool seamS = SEAM && (r0 > 0 || pery), seamN = SEAM && (r1 < ny || pery);
+    const int rstart = !SEAM && (r0 > 0 || pery) ? r0 - 1 : r0;
+    const int rend = !SEAM && (r1 < ny || pery) ? r1 : r1 - 1;
 
     // a non-positive dt leaves the state unchanged (runs past t_end)
     if (!(dt > 0.0)) {
@@ -523,29 +697,14 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
     const T rxv = SQ ? T(1) : rx, ryv = SQ ? T(1) : ry;
     const T tdt = T(dt);
     const T Mdx2 = pv.Mdx2T(), Mdy2 = pv.Mdy2T();
-    const T gam = T(a.gamma);
+    const T gam = T(a.gamma), gm1 = T(a.gamma - 1.0);
     const bool do_tvb = a.tvb_on, do_pp = a.pp_on;
     const T pp_eps = F32 ? T(a.pp_epsf) : T(a.pp_eps);
 
-    // FP32 state (plain or compensated): the per-cell wave speed and status
-    // tests of the epilogue run in FP32 (GB300's FP64 pipe is 1/64 of its FP32
-    // rate), the column totals in compensated FP32 (TwoSum; a compensated
-    // state adds its lo parts into the error term), converted to FP64 once per
-    // warp
-    constexpr bool F32R = sizeof(T) == 4;
-    T cs_hi[NV], cs_lo[NV];
-    T red_maxT = T(0);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) cs_hi[v] = cs_lo[v] = T(0);
     const double adv_speed = PHYS == PHYS_EULER ? 0.0 : pv.adv_speed();
-
-    // reduction accumulators (FP64)
-    double red_max = 0.0;
-    double red_sum[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) red_sum[v] = 0.0;
+    CellRed<T, NV> red;
     unsigned red_trouble = 0;
-    unsigned status = 0;
+    const Seam<T, K, B, PHYS, DEV> sc(pv.seam(), S, nx, LIM && a.limit);
 
     // limiter: rolling neighbour averages of this column
     T avg_prev[NV], avg_next[NV];
@@ -601,11 +760,13 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
     const double mlp_scale = a.M * hh_ * hh_;
 
     for (int r = rstart; r <= rend; ++r) {
-        const int ry_ = r < 0 ? r + ny : (r >= ny ? r - ny : r);
-        const bool out_row = r >= r0 && r < r1;
+        const int ry_ = SEAM ? r : (r < 0 ? r + ny : (r >= ny ? r - ny : r));
+        const bool out_row = SEAM || (r >= r0 && r < r1);
         const bool south_bc = (r == 0) && !pery;
-        const bool do_south = (r > rstart) || south_bc;   // flux through this row's south face
-        const bool keep_north = r < rend || (r == ny - 1 && !pery && out_row);
+        const bool do_south = r > rstart || south_bc;   // flux through this row's south face
+        const bool seam_row = SEAM && r == r0 && seamS; // its update waits for the seam below it
+        const bool last = r == rend;
+        const bool keep_north = SEAM ? !last || !seamN : (!last || (r == ny - 1 && !pery && out_row));
 
         // ---- load u^n (and limit on load) -------------------------------------
         T un[NV][NM];
@@ -694,17 +855,13 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
         }
 
         // ---- stages ---------------------------------------------------------------
-        T Vr[CRK_V_SMEM ? 1 : NV][CRK_V_SMEM ? 1 : NM];   // sum_i b_i * volume term (registers)
-        auto V = [&](int v, int m) -> T& {
-            if constexpr (CRK_V_SMEM) return slot(offV + v * NM + m);
-            else return Vr[v][m];
-        };
+        T V[NV][NM];      // sum_i b_i * volume term
         T FE[NQ][NV];     // sum_i b_i fhat on the east face
         T FS[NQ][NV];     // sum_i b_i fhat on the south face
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
-            for (int m = 0; m < NM; ++m) V(v, m) = T(0);
+            for (int m = 0; m < NM; ++m) V[v][m] = T(0);
 #pragma unroll
         for (int p = 0; p < NQ; ++p)
 #pragma unroll
@@ -861,12 +1018,12 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
 #pragma unroll
                     for (int v = 0; v < NV; v += 2)
 #pragma unroll
-                        for (int m = 0; m < NM; ++m) pfma(V(v, m), V(v + 1, m), vol[v][m], vol[v + 1][m], bi);
+                        for (int m = 0; m < NM; ++m) pfma(V[v][m], V[v + 1][m], vol[v][m], vol[v + 1][m], bi);
                 } else {
 #pragma unroll
                     for (int v = 0; v < NV; ++v)
 #pragma unroll
-                        for (int m = 0; m < NM; ++m) V(v, m) += bi * vol[v][m];
+                        for (int m = 0; m < NM; ++m) V[v][m] += bi * vol[v][m];
                 }
             }
             // face traces.  phi_m(-1, eta) = (-1)^i phi_m(1, eta): the east and
@@ -911,17 +1068,6 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
                     tE[p][v] = e; tW[p][v] = ww; tN[p][v] = n; tS[p][v] = s;
                 }
             }
-            // east/south Lax--Friedrichs fluxes formed inside the local operator's
-            // point loop (boundary strips and rows keep the separate path below)
-            const bool fuseE = CRK_LF_REUSE && need_L && need_flux && out_row && !has_bcW && !has_bcE;
-            const bool fuseS = CRK_LF_REUSE && need_L && need_flux && do_south && !south_bc;
-            T tWn[NQ][NV];
-            if (fuseE) {
-#pragma unroll
-                for (int p = 0; p < NQ; ++p)
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) tWn[p][v] = shfl_down(tW[p][v], 1);
-            }
             // local operator L_i = cm (face_loc - vol), eq. (2.7)
             if (need_L) {
                 T floc[NV][NM];
@@ -932,36 +1078,10 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
 #pragma unroll
                 for (int p = 0; p < NQ; ++p) {
                     T fe[NV], fw[NV], fn[NV], fs[NV];
-                    const T sE = ph.template fluxn<0>(tE[p], fe);
-                    const T sW = ph.template fluxn<0>(tW[p], fw);
-                    const T sN = ph.template fluxn<1>(tN[p], fn);
-                    const T sS = ph.template fluxn<1>(tS[p], fs);
-                    if (fuseE) {   // own east trace vs. the right lane's west trace
-                        T fwn[NV], F[NV];
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) fwn[v] = shfl_down(fw[v], 1);
-                        const T sWn = shfl_down(sW, 1);
-                        lf_from_fluxes<T, NV>(tE[p], fe, sE, tWn[p], fwn, sWn, F);
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) FE[p][v] += bi * F[v];
-                    }
-                    if (fuseS) {   // the row below's north trace vs. own south trace
-                        T lo[NV], flo[NV], F[NV];
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) {
-                            lo[v] = slot(offN + (i * NQ + p) * NV + v);
-                            flo[v] = slot(offNF + (i * NQ + p) * (NV + 1) + v);
-                        }
-                        const T slo = slot(offNF + (i * NQ + p) * (NV + 1) + NV);
-                        lf_from_fluxes<T, NV>(lo, flo, slo, tS[p], fs, sS, F);
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) FS[p][v] += bi * F[v];
-                    }
-                    if (CRK_LF_REUSE && keep_north) {
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) slot(offNF + (i * NQ + p) * (NV + 1) + v) = fn[v];
-                        slot(offNF + (i * NQ + p) * (NV + 1) + NV) = sN;
-                    }
+                    ph.template fluxn<0>(tE[p], fe);
+                    ph.template fluxn<0>(tW[p], fw);
+                    ph.template fluxn<1>(tN[p], fn);
+                    ph.template fluxn<1>(tS[p], fs);
                     if constexpr (NV % 2 == 0) {
                         // pW = (-1)^i pE, pS = (-1)^j pN: fe pE - fw pW = pE (fe -+ fw)
 #pragma unroll
@@ -1007,8 +1127,8 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
             }
             if (!need_flux) continue;
             // east face: own east trace vs. the west trace of the lane to the right
-            if (out_row && !fuseE) {
-                T dcE[NV];   // DEV: east neighbour's base minus this cell's
+            if (out_row) {
+                T tWn[NQ][NV], dcE[NV];   // DEV: east neighbour's base minus this cell's
                 if constexpr (DEV) {
 #pragma unroll
                     for (int v = 0; v < NV; ++v) dcE[v] = shfl_down(cb[v], 1) - cb[v];
@@ -1085,11 +1205,11 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
                     T F[NV];
                     llf_ax<0, false>(ph, tE[p], tWn[p], F);
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) FE[p][v] += hbi * F[v];
+                    for (int v = 0; v < NV; ++v) FE[p][v] = fma(hbi, F[v], FE[p][v]);
                 }
             }
             // south face: north trace of the row below (stored) vs. own south trace
-            if (do_south && !fuseS) {
+            if (do_south) {
                 T lo[NQ][NV];
                 if (south_bc) {   // row 0 without periodic wrap: boundary data (one uniform branch per row)
                     cold_branch();
@@ -1115,116 +1235,42 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
                     T F[NV];
                     llf_ax<1, false>(ph, lo[p], tS[p], F);
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) FS[p][v] += hbi * F[v];
+                    for (int v = 0; v < NV; ++v) FS[p][v] = fma(hbi, F[v], FS[p][v]);
                 }
             }
+            // traces for the row above, or for the seams at the segment's ends
             if (keep_north) {
 #pragma unroll
                 for (int p = 0; p < NQ; ++p)
 #pragma unroll
                     for (int v = 0; v < NV; ++v) slot(offN + (i * NQ + p) * NV + v) = tN[p][v];
+            } else if (SEAM && outlane) {
+#pragma unroll
+                for (int p = 0; p < NQ; ++p)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) *sc.north(seg, (i * NQ + p) * NV + v, col) = tN[p][v];
+            }
+            if (SEAM && seam_row && outlane) {
+#pragma unroll
+                for (int p = 0; p < NQ; ++p)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) *sc.south(seg, (i * NQ + p) * NV + v, col) = tS[p][v];
             }
         }
 
         // ---- finish the row below: its north face is this row's south face --------
         auto finish = [&](T (&P)[NV][NM], int rw) {
-            // write u^{n+1} of row rw and accumulate the FP64 reductions
+            if (outlane)
+                store_cell<T, PHYS, NV, NM, COMP>(a, pv, uin, uout, plane, (size_t)rw * nx + col, P, rx, ry, gm1, gam,
+                                                  red);
+        };
+        // an update that a seam completes, left in the output buffer (COMP: in the hi planes)
+        auto leave = [&](const T (&P)[NV][NM], int rw) {
             if (!outlane) return;
-            const size_t o = (size_t)rw * nx + col;
-            if constexpr (F32R) {
-                T avl[NV];   // COMP: lo part of the new averages
-                if constexpr (COMP) {
-                    // P holds Delta: u^{n+1} = (hi + lo) + Delta, hi' + lo' by
-                    // TwoSum; P[v][0] becomes hi' of the average
-                    const size_t lo_off = (size_t)C::NDOF * plane;
 #pragma unroll
-                    for (int v = 0; v < NV; ++v)
+            for (int v = 0; v < NV; ++v)
 #pragma unroll
-                        for (int m = 0; m < NM; ++m) {
-                            const size_t ix = (size_t)(v * NM + m) * plane + o;
-                            const T hi = uin[ix], lo = uin[lo_off + ix];
-                            const T d = P[v][m] + lo;
-                            const T sum = hi + d;
-                            const T bv = sum - hi;
-                            const T err = (hi - (sum - bv)) + (d - bv);
-                            uout[ix] = sum;
-                            uout[lo_off + ix] = err;
-                            if (m == 0) {
-                                P[v][0] = sum;
-                                avl[v] = err;
-                            }
-                        }
-                } else {
-#pragma unroll
-                    for (int v = 0; v < NV; ++v)
-#pragma unroll
-                        for (int m = 0; m < NM; ++m) uout[(size_t)(v * NM + m) * plane + o] = P[v][m];
-                }
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {   // TwoSum: cs_hi + cs_lo += P[v][0] exactly
-                    const T x = P[v][0];
-                    const T sum = cs_hi[v] + x;
-                    const T bv = sum - cs_hi[v];
-                    cs_lo[v] += (cs_hi[v] - (sum - bv)) + (x - bv);
-                    if constexpr (COMP) cs_lo[v] += avl[v];
-                    cs_hi[v] = sum;
-                }
-                if constexpr (PHYS == PHYS_EULER) {
-                    const T ir = T(1) / P[0][0];
-                    const T w = P[1][0] * ir, vv = P[2][0] * ir;
-                    const T p = ph.gm1 * (P[3][0] - T(0.5) * (P[1][0] * w + P[2][0] * vv));
-                    const T c = sqrt(fmax(gam * p * ir, T(0)));
-                    const T sp = (fabs(w) + c) * rx + (fabs(vv) + c) * ry;
-                    if (!(P[0][0] > T(0)) || !(p > T(0))) status |= ST_NONPHYSICAL;
-                    if (!(sp == sp)) status |= ST_NAN;
-                    red_maxT = fmax(red_maxT, sp);
-                } else {
-                    if (!(P[0][0] == P[0][0])) status |= ST_NAN;
-                }
-                return;
-            }
-            double av[NV];
-            if constexpr (COMP) {
-                // P holds Delta: u^{n+1} = (hi + lo) + Delta, hi' + lo' by TwoSum
-                const size_t lo_off = (size_t)C::NDOF * plane;
-#pragma unroll
-                for (int v = 0; v < NV; ++v)
-#pragma unroll
-                    for (int m = 0; m < NM; ++m) {
-                        const size_t ix = (size_t)(v * NM + m) * plane + o;
-                        const T hi = uin[ix], lo = uin[lo_off + ix];
-                        const T d = P[v][m] + lo;
-                        const T sum = hi + d;
-                        const T bv = sum - hi;
-                        const T err = (hi - (sum - bv)) + (d - bv);
-                        uout[ix] = sum;
-                        uout[lo_off + ix] = err;
-                        if (m == 0) av[v] = double(sum) + double(err);
-                    }
-            } else {
-#pragma unroll
-                for (int v = 0; v < NV; ++v)
-#pragma unroll
-                    for (int m = 0; m < NM; ++m) uout[(size_t)(v * NM + m) * plane + o] = P[v][m];
-#pragma unroll
-                for (int v = 0; v < NV; ++v) av[v] = double(P[v][0]);
-            }
-#pragma unroll
-            for (int v = 0; v < NV; ++v) red_sum[v] += av[v];
-            double sp;
-            if constexpr (PHYS == PHYS_EULER) {
-                const double ir = 1.0 / av[0];
-                const double w = av[1] * ir, vv = av[2] * ir;
-                const double p = (a.gamma - 1.0) * (av[3] - 0.5 * (av[1] * w + av[2] * vv));
-                const double c = sqrt(fmax(a.gamma * p * ir, 0.0));
-                sp = (fabs(w) + c) / pv.dx() + (fabs(vv) + c) / pv.dy();
-                if (!(av[0] > 0.0) || !(p > 0.0)) status |= ST_NONPHYSICAL;
-                if (!(sp == sp)) status |= ST_NAN;
-            } else {
-                sp = adv_speed;
-                if (!(av[0] == av[0])) status |= ST_NAN;
-            }
-            red_max = fmax(red_max, sp);
+                for (int m = 0; m < NM; ++m) uout[(size_t)(v * NM + m) * plane + (size_t)rw * nx + col] = P[v][m];
         };
         if (do_south && r - 1 >= r0 && r - 1 < r1) {
             // DEV: FS is relative to this row's base; the row below takes it
@@ -1236,22 +1282,32 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
                 for (int v = 0; v < NV; ++v) dcS[v] = cS[v] - cb[v];
                 ph.template fluxn<1>(dcS, gS);
             }
-            T P[NV][NM];
-#pragma unroll
-            for (int v = 0; v < NV; ++v)
-#pragma unroll
-                for (int m = 0; m < NM; ++m) {
-                    T s = T(0);
+            if (SEAM && r - 1 == r0 && seamS) {   // the seam completes the row below: its north flux
+                if (outlane) {
 #pragma unroll
                     for (int p = 0; p < NQ; ++p)
-                        if (tb.pN[p][m] != 0.0) s += FS[p][v] * T(tb.pN[p][m]);
-                    if constexpr (DEV) {
-                        if (tb.sN[m] != 0.0) s -= gS[v] * T(tb.sN[m]);
-                    }
-                    P[v][m] = slot(offP + v * NM + m) - tdt * T(tb.cm[m]) * (ry * s);
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) *sc.flux(seg, p * NV + v, col) = FS[p][v];
+                    if constexpr (DEV)
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) *sc.flux(seg, NQ * NV + v, col) = gS[v];
                 }
-            finish(P, r - 1);
+            } else {
+                T P[NV][NM];
+#pragma unroll
+                for (int v = 0; v < NV; ++v)
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) P[v][m] = slot(offP + v * NM + m);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    T Fv[NQ];
+                    column<NQ, NV>(FS, v, Fv);
+                    add_north<T, K, B, DEV>(P[v], Fv, DEV ? gS[v] : T(0), ry, tdt);
+                }
+                finish(P, r - 1);
+            }
         }
+
         if (!out_row) continue;
 
         // ---- this row: east/west/south faces and the volume term ----------------------
@@ -1281,20 +1337,34 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
                 FEm[p][v] = FE[p][v] - FW[p][v];
                 FEp[p][v] = FE[p][v] + FW[p][v];
             }
-        T P[NV][NM];
+        T P[NV][NM];   // first the east/west face terms, then the update
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
             for (int m = 0; m < NM; ++m) {
-                T sx = T(0), sy = T(0);
+                T sx = T(0);
 #pragma unroll
-                for (int p = 0; p < NQ; ++p) {
-                    if (tb.pE[p][m] != 0.0) sx += (tb.ip[m] == 0 ? FEm[p][v] : FEp[p][v]) * T(tb.pE[p][m]);
-                    if (tb.pS[p][m] != 0.0) sy -= FS[p][v] * T(tb.pS[p][m]);
-                }
-                const T fsum = SQ ? fma(rx, sx + sy, -V(v, m)) : rx * sx + ry * sy - V(v, m);
-                P[v][m] = (COMP ? T(0) : un[v][m]) - tdt * T(tb.cm[m]) * fsum;
+                for (int p = 0; p < NQ; ++p)
+                    if (tb.pE[p][m] != 0.0) sx = fma(tb.ip[m] == 0 ? FEm[p][v] : FEp[p][v], T(tb.pE[p][m]), sx);
+                P[v][m] = sx;
             }
+        if (SEAM && seam_row) {
+            if (outlane)
+#pragma unroll
+                for (int v = 0; v < NV; ++v)
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) {
+                        *sc.vol(seg, v * NM + m, col) = V[v][m];
+                        if (LIM && a.limit) *sc.un(seg, v * NM + m, col) = un[v][m];
+                    }
+        } else {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                T Fv[NQ];
+                column<NQ, NV>(FS, v, Fv);
+                row_update<T, K, B, COMP, SQ>(P[v], P[v], V[v], Fv, un[v], rx, ry, tdt);
+            }
+        }
         if (r == ny - 1 && !pery) {
             // top boundary: north face flux from the stored north traces
             cold_branch();
@@ -1320,19 +1390,31 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
                     }, hi);
                     llf_ax<1>(ph, lo, hi, F);
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) FN[p][v] += bi * F[v];
+                    for (int v = 0; v < NV; ++v) FN[p][v] = fma(bi, F[v], FN[p][v]);
                 }
             }
+            if (SEAM && seam_row) {
+                if (outlane) {
 #pragma unroll
-            for (int v = 0; v < NV; ++v)
+                    for (int p = 0; p < NQ; ++p)
 #pragma unroll
-                for (int m = 0; m < NM; ++m) {
-                    T s = T(0);
+                        for (int v = 0; v < NV; ++v) *sc.flux(seg, p * NV + v, col) = FN[p][v];
+                    if constexpr (DEV)   // already relative to this row's base
 #pragma unroll
-                    for (int p = 0; p < NQ; ++p) s += FN[p][v] * T(tb.pN[p][m]);
-                    P[v][m] -= tdt * T(tb.cm[m]) * (ry * s);
+                        for (int v = 0; v < NV; ++v) *sc.flux(seg, NQ * NV + v, col) = T(0);
                 }
-            finish(P, r);
+                leave(P, r);
+            } else {
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    T Fv[NQ];
+                    column<NQ, NV>(FN, v, Fv);
+                    add_north<T, K, B, false>(P[v], Fv, T(0), ry, tdt);
+                }
+                finish(P, r);
+            }
+        } else if (SEAM && (seam_row || last)) {
+            leave(P, r);
         } else {
 #pragma unroll
             for (int v = 0; v < NV; ++v)
@@ -1341,20 +1423,16 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
         }
     }
 
-    // ---- FP64 reductions: warp -> per-warp slot -> finalize (batch: last warp) -------
-    const double cell = pv.cell();
-    if constexpr (F32R) {
-        red_max = PHYS == PHYS_EULER ? double(red_maxT) : (outlane && r0 < r1 ? adv_speed : 0.0);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) red_sum[v] = double(cs_hi[v]) + double(cs_lo[v]);
-    }
-    step_epilogue<NV, C::NRED>(a, pv, gw, lane, total_warps, red_max, red_sum, red_trouble, status, cell, t0, dt);
+    // ---- FP64 reductions: warp -> per-warp slot -> the launch that ends the step -----
+    red.template close<PHYS>(outlane && r0 < r1 ? adv_speed : 0.0);
+    step_epilogue<NV, C::NRED>(pv, gw, lane, red.max, red.sum, red_trouble, red.status);
 }
 
 // One problem: the launch arguments describe the mesh; dt and t come from
 // the arguments or from the device run state (device-driven runs).
+// (FP64 always leaves its seams to the seam launches: see use_seams)
 template <class T, int K, int B, int PHYS, bool COMP = false, bool MLPI = false, bool LIM = true, bool DEV = false,
-          bool SQ = false>
+          bool SQ = false, bool SEAM = sizeof(T) == 8>
 __global__ void __launch_bounds__(CRK_STEP_MAXT, PHYS == PHYS_ADV ? CRK_STEP_MINB_ADV : CRK_STEP_MINB2)
     step2d_kernel(const StepArgs a) {
     if constexpr (MLPI) {
@@ -1367,28 +1445,257 @@ __global__ void __launch_bounds__(CRK_STEP_MAXT, PHYS == PHYS_ADV ? CRK_STEP_MIN
     const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (gw >= a.n_strips * a.n_segs) return;   // whole warp leaves; no block barriers
     const ArgsView<T> pv{a, a.dt_from_dev ? a.ds->t : a.t, a.dt_from_dev ? a.ds->dt : a.dt};
-    step2d_body<T, K, B, PHYS, COMP, MLPI, LIM, DEV, SQ>(a, pv, gw);
+    step2d_body<T, K, B, PHYS, COMP, MLPI, LIM, DEV, SQ, SEAM>(a, pv, gw);
+}
+
+template <class T>
+constexpr int SEAM_THREADS = sizeof(T) == 4 ? SEAM_THREADS_F32 : SEAM_THREADS_F64;
+
+// The step's second launch: the fluxes sum_i b_i fhat of the seams, one thread
+// per (seam, face point, column), columns fastest, all stages' traces loaded
+// before they are used.  DEV: relative to the upper row's base; the move to
+// the lower row's is stored with it.  (One thread per cell forming the fluxes
+// of its own seams and completing the cell did them twice and in fewer threads:
+// 0.151 ms against 0.054 + 0.048 for FP64 P^2 on 640 x 160, 0.086 against 0.018 +
+// 0.019 for Q^2 RK4 on 80 x 80.)
+template <class T, int K, int B, int PHYS, bool DEV, class PV>
+__device__ __forceinline__ void seam_flux_body(const StepArgs& a, const PV& pv, int id, bool limited) {
+    using C = Step2D<T, K, B, PHYS>;
+    constexpr int NQ = C::NQ, NV = C::NV;
+    const int nx = pv.nx(), ny = pv.ny(), nseg = pv.n_segs(), S = a.s;
+    const int row = id / nx, col = id - row * nx;
+    const int s = row / NQ, p = row - s * NQ;   // the seam below segment s
+    if (s >= nseg || !(pv.dt() > 0.0)) return;
+    if (s == 0 && a.bc[2].type != BC_PERIODIC) return;
+    const int sl = s > 0 ? s - 1 : nseg - 1;
+    const Seam<T, K, B, PHYS, DEV> sc(pv.seam(), S, nx, limited);
+    std::conditional_t<DEV, EulerDev<T>, Phys<T, PHYS>> ph;
+    if constexpr (PHYS == PHYS_EULER) {
+        ph.gamma = T(a.gamma);
+        ph.gm1 = T(a.gamma - 1.0);
+    } else {
+        ph.bx = T(a.beta[0]);
+        ph.by = T(a.beta[1]);
+    }
+    T lo[MAXS][NV], hi[MAXS][NV], bs[MAXS];
+#pragma unroll
+    for (int i = 0; i < MAXS; ++i) {
+        bs[i] = i < S ? tab_bT<T>(a, i) : T(0);
+        if (bs[i] != T(0))
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                lo[i][v] = *sc.north(sl, (i * NQ + p) * NV + v, col);
+                hi[i][v] = *sc.south(s, (i * NQ + p) * NV + v, col);
+            }
+    }
+    T dc[NV], gS[NV];
+    if constexpr (DEV) {
+        const size_t plane = (size_t)nx * ny;
+        const int ru = seg_row(s, ny, nseg), rl = ru > 0 ? ru - 1 : ny - 1;
+        const T* __restrict__ uin = pv.uin();
+        T cu[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            cu[v] = uin[(size_t)(v * C::NM) * plane + (size_t)ru * nx + col];
+            dc[v] = uin[(size_t)(v * C::NM) * plane + (size_t)rl * nx + col] - cu[v];
+        }
+        ph.set_base(cu);
+        if (p == 0) {
+            ph.template fluxn<1>(dc, gS);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) *sc.below(s, NQ * NV + v, col) = gS[v];
+        }
+    }
+    T F[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) F[v] = T(0);
+#pragma unroll
+    for (int i = 0; i < MAXS; ++i) {
+        if (bs[i] == T(0)) continue;
+        const T hbi = T(0.5) * bs[i];
+        if constexpr (DEV)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) lo[i][v] += dc[v];
+        T G[NV];
+        llf_ax<1, false>(ph, lo[i], hi[i], G);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) F[v] = fma(hbi, G[v], F[v]);
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) *sc.below(s, p * NV + v, col) = F[v];
+}
+
+template <class T, int K, int B, int PHYS, bool DEV>
+__global__ void __launch_bounds__(SEAM_THREADS<T>) seam_flux_kernel(const StepArgs a, bool limited) {
+    wait_for_step();
+    allow_dependent_launch();
+    const ArgsView<T> pv{a, a.dt_from_dev ? a.ds->t : a.t, a.dt_from_dev ? a.ds->dt : a.dt};
+    seam_flux_body<T, K, B, PHYS, DEV>(a, pv, blockIdx.x * SEAM_THREADS<T> + threadIdx.x, limited);
+}
+
+// The third launch: one thread per variable of a cell of a segment's first or
+// last row completes it: a warp per 32 cells (columns fastest) and variable, so
+// that a thread holds a quarter of a cell's loads and registers; the averages
+// meet in shared memory for the wave speed.  Block blk of nblk takes its share of
+// the cells and of the step warps' slots; the last block to arrive (an atomic
+// counter, no waiting) reduces the blocks' slots in a fixed order and updates
+// the run state.  At most two blocks per SM (seam_blocks): a block per 32 cells
+// took longer wherever they were many (FP32 P^2 on 1920 x 480 in segments of 4
+// rows, 4 steps: 1.46 against 1.29 ms: FP64 block reductions and the counter).
+template <class T, int K, int B, int PHYS, bool COMP, bool DEV, bool SQ, class PV>
+__device__ __forceinline__ void seam_body(const StepArgs& a, const PV& pv, int blk, int nblk) {
+    using C = Step2D<T, K, B, PHYS>;
+    constexpr int NQ = C::NQ, NM = C::NM, NV = C::NV, NT = SEAM_CELL_THREADS, G = NT / (32 * NV);
+    __shared__ T avg[G][NV][32];
+    const double dt = pv.dt();
+    if (!(dt > 0.0)) return;   // the step left the state and the run state unchanged
+    const int nx = pv.nx(), ny = pv.ny(), nseg = pv.n_segs();
+    const size_t plane = (size_t)nx * ny;
+    const bool pery = a.bc[2].type == BC_PERIODIC, limited = !COMP && a.limit;
+    const Seam<T, K, B, PHYS, DEV> sc(pv.seam(), a.s, nx, limited);
+    const T rx = pv.rxT(), ry = pv.ryT(), tdt = T(dt);
+    T gam, gm1;
+    if constexpr (sizeof(T) == 4) {
+        gam = a.gammaf;
+        gm1 = a.gm1f;
+    } else {
+        gam = a.gamma;
+        gm1 = a.gamma - 1.0;
+    }
+    const T* __restrict__ uin = pv.uin();
+    T* __restrict__ uout = pv.uout();
+    const int lane = threadIdx.x & 31, v = (threadIdx.x >> 5) % NV, grp = threadIdx.x / (32 * NV);
+    const int both = nseg != ny;   // cells by (segment, first or last row, column), or (segment, column)
+    const int groups = (int)(((long long)nx * nseg * (1 + both) + 31) / 32);
+    T hi = T(0), lo = T(0), fastest = T(0);   // total of this thread's variable, hi + lo
+    unsigned st = 0;
+    for (int base = blk * G; base < groups; base += nblk * G) {
+        const int cell = (base + grp) * 32 + lane;
+        const int row = cell / nx, col = cell - row * nx, seg = row >> both;
+        bool wrote = false;
+        if (seg < nseg) {
+            const int r0 = seg_row(seg, ny, nseg), r1 = seg_row(seg + 1, ny, nseg);
+            const bool top = both && (row & 1), one = r1 - r0 == 1;
+            // the faces the row waits for: below a first row, above a last one
+            const bool south = !top && (seg > 0 || pery), north = (top || one) && (seg + 1 < nseg || pery);
+            wrote = top ? north && !one : south || north;
+            if (wrote) {
+                const size_t o = (size_t)(top ? r1 - 1 : r0) * nx + col;
+                T P[NM], V[NM], un[NM], FS[NQ], FN[NQ];
+                T gS = T(0);
+#pragma unroll
+                for (int m = 0; m < NM; ++m) P[m] = uout[(size_t)(v * NM + m) * plane + o];
+                // the north face: the seam above, or the flux the step formed
+                const int su = seg + 1 < nseg ? seg + 1 : 0;
+#pragma unroll
+                for (int p = 0; p < NQ; ++p)
+                    FN[p] = north ? *sc.below(su, p * NV + v, col) : *sc.flux(seg, p * NV + v, col);
+                if constexpr (DEV) gS = north ? *sc.below(su, NQ * NV + v, col) : *sc.flux(seg, NQ * NV + v, col);
+                if (south) {
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) {
+                        V[m] = *sc.vol(seg, v * NM + m, col);
+                        if constexpr (COMP) un[m] = T(0);
+                        else un[m] = limited ? *sc.un(seg, v * NM + m, col) : uin[(size_t)(v * NM + m) * plane + o];
+                    }
+#pragma unroll
+                    for (int p = 0; p < NQ; ++p) FS[p] = *sc.below(seg, p * NV + v, col);
+                    row_update<T, K, B, COMP, SQ>(P, P, V, FS, un, rx, ry, tdt);
+                }
+                add_north<T, K, B, DEV>(P, FN, gS, ry, tdt);
+                T al = T(0);
+#pragma unroll
+                for (int m = 0; m < NM; ++m) {
+                    const size_t ix = (size_t)(v * NM + m) * plane + o;
+                    if constexpr (COMP) {
+                        T h, l;
+                        store_comp(uin, uout, ix, (size_t)(NV * NM) * plane, P[m], h, l);
+                        if (m == 0) {
+                            P[0] = h;
+                            al = l;
+                        }
+                    } else {
+                        uout[ix] = P[m];
+                    }
+                }
+                avg[grp][v][lane] = P[0];
+                const T sum = hi + P[0];   // TwoSum
+                const T bv = sum - hi;
+                lo += (hi - (sum - bv)) + (P[0] - bv);
+                if constexpr (COMP) lo += al;
+                hi = sum;
+            }
+        }
+        __syncthreads();
+        if (v == 0 && wrote) {
+            T A[NV];
+#pragma unroll
+            for (int i = 0; i < NV; ++i) A[i] = avg[grp][i][lane];
+            fastest = fmax(fastest, new_speed<T, PHYS, NV>(a, pv, A, rx, ry, gm1, gam, st));
+        }
+        __syncthreads();
+    }
+    DevState* ds = pv.ds();
+    st = __reduce_or_sync(0xffffffffu, st);
+    if (lane == 0 && st) atomicOr(&ds->status, st);
+    StepRed<NV> sr;
+    sr.key = speed_key(double(fastest));
+    const double total = double(hi) + double(lo);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) sr.sum[i] = i == v ? total : 0.0;
+    // the block's slot: its cells, and its share of the step warps' slots
+    const int nw = pv.total_warps();
+    for (int w = blk * NT + threadIdx.x; w < nw; w += nblk * NT) sr.add_slot(pv.partials() + (size_t)w * C::NRED);
+    sr.template block_reduce<NT>();
+    double* const slots = pv.partials() + (size_t)nw * C::NRED;
+    unsigned prev = 0;
+    if (threadIdx.x == 0) {
+        sr.put_slot(slots + (size_t)blk * C::NRED);
+        __threadfence();
+        prev = atomicAdd(&ds->counter, 1u);
+    }
+    if (!__syncthreads_or(threadIdx.x == 0 && prev == (unsigned)nblk - 1)) return;
+    __threadfence();
+    StepRed<NV> tot;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nblk; b += NT) tot.add_slot(slots + (size_t)b * C::NRED);
+    tot.template block_reduce<NT>();
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < NV; ++i) tot.sum[i] *= pv.cell();
+        finish_run_state(a, ds, __longlong_as_double((long long)tot.key), tot.sum, NV, double(tot.trouble), pv.t(),
+                         dt, ds->cfl, ds->t_end, ds->lim_count, pv.cur(), pv.done());
+    }
+}
+
+template <class T, int K, int B, int PHYS, bool COMP, bool DEV, bool SQ>
+__global__ void __launch_bounds__(SEAM_CELL_THREADS) seam_kernel(const StepArgs a) {
+    wait_for_step();
+    const ArgsView<T> pv{a, a.dt_from_dev ? a.ds->t : a.t, a.dt_from_dev ? a.ds->dt : a.dt};
+    seam_body<T, K, B, PHYS, COMP, DEV, SQ>(a, pv, blockIdx.x, gridDim.x);
+}
+
+// launches of the seams after a single-problem step launched with b
+template <class T, int K, int B, int PHYS, bool COMP = false, bool DEV = false, bool SQ = false>
+inline cudaError_t launch_seam(const StepArgs& b, cudaStream_t st) {
+    const cudaError_t e = launch_dependent(&seam_flux_kernel<T, K, B, PHYS, DEV>,
+                                           seam_flux_blocks(sizeof(T), K + 1, b.nx, b.n_segs), SEAM_THREADS<T>, st, b,
+                                           !COMP && b.limit);
+    if (e != cudaSuccess) return e;
+    return launch_dependent(&seam_kernel<T, K, B, PHYS, COMP, DEV, SQ>, seam_blocks(Step2D<T, K, B, PHYS>::NV, b.nx, b.ny, b.n_segs, 2 * std::max(1, sm_count())), SEAM_CELL_THREADS,
+                            st, b);
 }
 
 // Batched ensemble: problems of different sizes and domains share the
 // scheme, tableau and boundary types; each has its own state slice, run state
 // (t, dt from its own FP64 wave-speed reduction, t_end, status) and buffer
-// index.  Warps take (problem, warp) tasks from a flattened table.  A problem
-// whose dt is 0 (it reached t_end) costs nothing: its warps return at once.
-// SQ: problems with square cells (pb.sq) take the square-cell form of the
-// step (a branch per task, uniform over the warp), the others the general one.
-
-template <class T, int K, int B, int PHYS, bool LIM = true, bool SQ = false>
-__global__ void __launch_bounds__(256) batch_step2d_kernel(const StepArgs a, const BatchProblem* __restrict__ probs,
-                                                           const int2* __restrict__ tasks, int n_tasks,
-                                                           DevState* states, int* curs, unsigned* done,
-                                                           const T* bufA, T* bufB) {
-    const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (gw >= n_tasks) return;
-    const int2 tk = tasks[gw];
-    const BatchProblem pb = probs[tk.x];
-    DevState* ds = states + tk.x;
-    const int cur = curs[tk.x];
+// index.  Warps take (problem, warp) tasks from a flattened table; one block per
+// problem ends its step.  A problem whose dt is 0 (it reached t_end) costs
+// nothing: its warps return at once.
+template <class T, int K, int B, int PHYS>
+__device__ __forceinline__ ProbView<T> problem_view(const StepArgs& a, const BatchProblem& pb, int p, DevState* states,
+                                                    int* curs, unsigned* done, const T* bufA, T* bufB) {
+    DevState* ds = states + p;
+    const int cur = curs[p];
     ProbView<T> pv;
     T* A = const_cast<T*>(bufA) + pb.offset;
     T* Bb = bufB + pb.offset;
@@ -1411,17 +1718,92 @@ __global__ void __launch_bounds__(256) batch_step2d_kernel(const StepArgs a, con
     pv.n_segs_ = pb.n_segs;
     pv.seg_len_ = a.seg_len;
     pv.total_warps_ = pb.n_strips * pb.n_segs;
-    pv.partials_ = a.partials + (size_t)pb.warp0 * Step2D<T, K, B, PHYS>::NRED;
+    pv.partials_ = a.partials + (size_t)pb.slot0 * Step2D<T, K, B, PHYS>::NRED;
+    pv.seam_ = static_cast<T*>(a.seam) + pb.seam0;
     pv.ds_ = ds;
-    pv.cur_ = curs + tk.x;
+    pv.cur_ = curs + p;
     pv.done_ = done;
+    return pv;
+}
+
+// SQ: problems with square cells (pb.sq) take the square-cell form of the
+// step (a branch per task, uniform over the warp), the others the general one.
+template <class T, int K, int B, int PHYS, bool LIM = true, bool SQ = false, bool SEAM = sizeof(T) == 8>
+__global__ void __launch_bounds__(256) batch_step2d_kernel(const StepArgs a, const BatchProblem* __restrict__ probs,
+                                                           const int2* __restrict__ tasks, int n_tasks,
+                                                           DevState* states, int* curs, unsigned* done,
+                                                           const T* bufA, T* bufB) {
+    allow_dependent_launch();
+    const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (gw >= n_tasks) return;
+    const int2 tk = tasks[gw];
+    const BatchProblem pb = probs[tk.x];
+    const ProbView<T> pv = problem_view<T, K, B, PHYS>(a, pb, tk.x, states, curs, done, bufA, bufB);
     if constexpr (SQ) {
         if (pb.sq) {
-            step2d_body<T, K, B, PHYS, false, false, LIM, false, true>(a, pv, tk.y);
+            step2d_body<T, K, B, PHYS, false, false, LIM, false, true, SEAM>(a, pv, tk.y);
             return;
         }
     }
-    step2d_body<T, K, B, PHYS, false, false, LIM, false, false>(a, pv, tk.y);
+    step2d_body<T, K, B, PHYS, false, false, LIM, false, false, SEAM>(a, pv, tk.y);
+}
+
+// The seams of a batched step: blocks of (problem, block) from two tables
+template <class T, int K, int B, int PHYS>
+__global__ void __launch_bounds__(SEAM_THREADS<T>)
+    batch_seam_flux_kernel(const StepArgs a, const BatchProblem* __restrict__ probs, const int2* __restrict__ tasks,
+                           DevState* states, int* curs, unsigned* done, const T* bufA, T* bufB, bool limited) {
+    const int2 tk = tasks[blockIdx.x];   // the tables are constant
+    const BatchProblem pb = probs[tk.x];
+    wait_for_step();
+    allow_dependent_launch();
+    const ProbView<T> pv = problem_view<T, K, B, PHYS>(a, pb, tk.x, states, curs, done, bufA, bufB);
+    seam_flux_body<T, K, B, PHYS, false>(a, pv, tk.y * SEAM_THREADS<T> + threadIdx.x, limited);
+}
+
+// SQ: problems with square cells (pb.sq) took the square-cell form of the step
+template <class T, int K, int B, int PHYS, bool SQ>
+__global__ void __launch_bounds__(SEAM_CELL_THREADS)
+    batch_seam_kernel(const StepArgs a, const BatchProblem* __restrict__ probs, const int2* __restrict__ tasks,
+                      DevState* states, int* curs, unsigned* done, const T* bufA, T* bufB) {
+    const int2 tk = tasks[blockIdx.x];
+    const BatchProblem pb = probs[tk.x];
+    wait_for_step();
+    const ProbView<T> pv = problem_view<T, K, B, PHYS>(a, pb, tk.x, states, curs, done, bufA, bufB);
+    if constexpr (SQ) {
+        if (pb.sq) {
+            seam_body<T, K, B, PHYS, false, false, true>(a, pv, tk.y, pb.n_seam_blocks);
+            return;
+        }
+    }
+    seam_body<T, K, B, PHYS, false, false, false>(a, pv, tk.y, pb.n_seam_blocks);
+}
+
+// The end of a batched step without seams: one block per problem reduces its
+// slots and updates its run state and buffer index
+constexpr int BATCH_FINALIZE_THREADS = 128;
+template <int NV>
+__global__ void __launch_bounds__(BATCH_FINALIZE_THREADS)
+    batch_finalize_kernel(const StepArgs a, const BatchProblem* __restrict__ probs, DevState* states, int* curs,
+                          unsigned* done) {
+    const int p = blockIdx.x;
+    const long long slot0 = probs[p].slot0;
+    const int total = probs[p].n_strips * probs[p].n_segs;
+    const double cell = probs[p].dx * probs[p].dy;
+    wait_for_step();
+    DevState* ds = states + p;
+    const double dt = ds->dt;
+    if (!(dt > 0.0)) return;   // the problem has reached t_end
+    StepRed<NV> red;
+#pragma unroll 4
+    for (int w = threadIdx.x; w < total; w += BATCH_FINALIZE_THREADS)
+        red.add_slot(a.partials + (size_t)(slot0 + w) * (NV + 2));
+    red.template block_reduce<BATCH_FINALIZE_THREADS>();
+    if (threadIdx.x == 0) {
+        for (int v = 0; v < NV; ++v) red.sum[v] *= cell;
+        finish_run_state(a, ds, __longlong_as_double((long long)red.key), red.sum, NV, double(red.trouble), ds->t, dt,
+                         ds->cfl, ds->t_end, ds->lim_count, curs + p, done);
+    }
 }
 
 }  // namespace crk

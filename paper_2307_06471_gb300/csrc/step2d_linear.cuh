@@ -82,7 +82,6 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
     const T* __restrict__ uin = static_cast<const T*>(a.uin);
     T* __restrict__ uout = static_cast<T*>(a.uout);
     const double dt = pv.dt();
-    const double t0 = pv.t();
 
     const int strip = gw % a.n_strips;
     const int seg = gw / a.n_strips;
@@ -294,7 +293,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
 
     double red_max = (outlane && r0 < r1) ? a.adv_speed : 0.0;
     double red_sum[1] = {double(cs_hi) + double(cs_lo)};
-    step_epilogue<1, 3>(a, pv, gw, lane, total_warps, red_max, red_sum, 0u, status, a.cell, t0, dt);
+    step_epilogue<1, 3>(pv, gw, lane, red_max, red_sum, 0u, status);
 }
 
 }  // namespace crk
