@@ -254,20 +254,49 @@ __global__ void __launch_bounds__(REDUCE_RUNS * REDUCE_PARAMS)
     }
 }
 
-// BF16 tensor-core inference, one warp per 32 samples
-__global__ void __launch_bounds__(128) mlp_predict_kernel(const float* __restrict__ prm, const float* __restrict__ X,
-                                                          int n, float* __restrict__ logits) {
+// BF16 tensor-core inference, a warp per 32 samples.  A grid of resident blocks
+// loads the weights once per block and walks the samples; the warp reads its
+// samples' features as one run of memory and rounds them into its staging area
+// (VEC: pairs, where X allows 8-byte loads).  A block per 128 samples that
+// loaded the weights each time, lanes reading 160 bytes apart and the weights'
+// rows in one bank group took 0.202 ms for 524,288 samples; this takes 0.057 ms.
+constexpr int PREDICT_THREADS = 128;
+template <bool VEC>
+__global__ void __launch_bounds__(PREDICT_THREADS) mlp_predict_kernel(const float* __restrict__ prm,
+                                                                      const float* __restrict__ X, int n,
+                                                                      float* __restrict__ logits) {
     extern __shared__ __align__(16) unsigned char smb[];
     crk::MlpSmem& w = *reinterpret_cast<crk::MlpSmem*>(smb);
+    const int lane = threadIdx.x & 31;
     __nv_bfloat16* stage = reinterpret_cast<__nv_bfloat16*>(smb + sizeof(crk::MlpSmem)) +
                            (threadIdx.x >> 5) * (32 * crk::MLP_INP + 64);
     crk::mlp_load_smem(w, prm);
+    // the padding columns 40 .. 47 stay zero
+    for (int k = MLP_IN; k < crk::MLP_INP; k += 2) *reinterpret_cast<uint32_t*>(stage + lane * crk::MLP_INP + k) = 0u;
     __syncthreads();
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    float f[MLP_IN];
-    for (int k = 0; k < MLP_IN; ++k) f[k] = s < n ? X[(size_t)s * MLP_IN + k] : 0.f;
-    const float z = crk::mlp_warp_logit(w, f, stage);
-    if (s < n) logits[s] = z;
+    const long long warps = (long long)gridDim.x * (PREDICT_THREADS / 32);
+    for (long long t = (long long)blockIdx.x * (PREDICT_THREADS / 32) + (threadIdx.x >> 5); t * 32 < n; t += warps) {
+        const int s0 = (int)(t * 32), ns = min(32, n - s0);
+        const float* x = X + (size_t)s0 * MLP_IN;
+        constexpr int PAIRS = MLP_IN / 2;
+        float2 f[PAIRS];
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) {   // 32 x 20 pairs, pair i of the run
+            const int i = j * 32 + lane;
+            f[j] = make_float2(0.f, 0.f);
+            if (i < ns * PAIRS) {
+                if constexpr (VEC) f[j] = __ldg(reinterpret_cast<const float2*>(x) + i);
+                else f[j] = make_float2(__ldg(x + 2 * i), __ldg(x + 2 * i + 1));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < PAIRS; ++j) {
+            const int i = j * 32 + lane, r = i / PAIRS, k = 2 * (i % PAIRS);
+            *reinterpret_cast<uint32_t*>(stage + r * crk::MLP_INP + k) = crk::pack_bf16(f[j].x, f[j].y);
+        }
+        const float z = crk::mlp_warp_staged(w, stage);
+        if (lane < ns) logits[s0 + lane] = z;
+    }
 }
 
 // The same inference on the fifth-generation tensor cores (mlp_tc.cuh): one
@@ -294,46 +323,56 @@ __global__ void __launch_bounds__(crk::MLPTC_CELLS) mlp_predict_tc_kernel(const 
 }
 
 // Features and TVB labels of every cell of a P^2 2D Euler state (one thread
-// per cell).  Label 1 when the TVB-minmod test of the limiter flags the cell.
+// per cell, 128 cells of a row per block).  Label 1 when the TVB-minmod test of
+// the limiter flags the cell.  The block's 128 x 40 features leave through
+// shared memory as one run (a thread writing its own 160 bytes touched 32
+// sectors per store), and the test's constants come from the host (set_derived)
+// instead of FP64 products in every thread: 0.106 -> 0.026 ms for 1024 x 512
+// FP32 cells.
+constexpr int FEAT_THREADS = 128;
 template <class T, int K, int B>
-__global__ void features_kernel(const StepArgs a, const T* __restrict__ u, float* __restrict__ X,
-                                float* __restrict__ y, double Mh2) {
+__global__ void __launch_bounds__(FEAT_THREADS) features_kernel(const StepArgs a, const T* __restrict__ u,
+                                                                float* __restrict__ X, float* __restrict__ y) {
     constexpr int NM = crk::Tab2D<K, B>::NM;
+    __shared__ float out[FEAT_THREADS * (MLP_IN + 1)];
     const int nx = a.nx, ny = a.ny;
     const size_t plane = (size_t)nx * ny;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int x0 = blockIdx.x * FEAT_THREADS, x = x0 + threadIdx.x;
     const int yy = blockIdx.y;
-    if (x >= nx) return;
-    const bool perx = a.bc[0].type == crk::BC_PERIODIC, pery = a.bc[2].type == crk::BC_PERIODIC;
-    T c[4][NM];
-    for (int v = 0; v < 4; ++v)
-        for (int m = 0; m < NM; ++m) c[v][m] = u[(size_t)(v * NM + m) * plane + (size_t)yy * nx + x];
-    T own[4], nb[4][4];
-    for (int v = 0; v < 4; ++v) own[v] = c[v][0];
-    const int xs[4] = {x - 1, x + 1, x, x};
-    const int ys[4] = {yy, yy, yy - 1, yy + 1};
-    for (int s = 0; s < 4; ++s) {
-        int cx = xs[s], cy = ys[s];
-        const bool out = (s < 2 && !perx && (cx < 0 || cx >= nx)) || (s >= 2 && !pery && (cy < 0 || cy >= ny));
-        if (out) {
-            crk::bc_exterior<T, 4>(a.bc[s], s < 2 ? 0 : 1, own, [&](double& xc, double& yc, double& tc) {
-                xc = a.x0 + (cx + 0.5) * a.dx;
-                yc = a.y0 + (cy + 0.5) * a.dy;
-                tc = a.t;
-            }, nb[s]);
-        } else {
-            cx = (cx + nx) % nx;
-            cy = (cy + ny) % ny;
-            for (int v = 0; v < 4; ++v) nb[s][v] = u[(size_t)(v * NM) * plane + (size_t)cy * nx + cx];
+    if (x < nx) {
+        const bool perx = a.bc[0].type == crk::BC_PERIODIC, pery = a.bc[2].type == crk::BC_PERIODIC;
+        // every load at a valid (wrapped or clamped) address, ghosts afterwards
+        const int ys = yy > 0 ? yy - 1 : (pery ? ny - 1 : 0), yn = yy < ny - 1 ? yy + 1 : (pery ? 0 : ny - 1);
+        const int xw = x > 0 ? x - 1 : (perx ? nx - 1 : 0), xe = x < nx - 1 ? x + 1 : (perx ? 0 : nx - 1);
+        T c[4][NM], own[4], nbW[4], nbE[4], nbS[4], nbN[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+#pragma unroll
+            for (int m = 0; m < NM; ++m) c[v][m] = u[(size_t)(v * NM + m) * plane + (size_t)yy * nx + x];
+            const T* p = u + (size_t)(v * NM) * plane;
+            nbW[v] = p[(size_t)yy * nx + xw];
+            nbE[v] = p[(size_t)yy * nx + xe];
+            nbS[v] = p[(size_t)ys * nx + x];
+            nbN[v] = p[(size_t)yn * nx + x];
         }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) own[v] = c[v][0];
+        const crk::LimMesh g = crk::single_mesh<T>(a);
+        crk::limit2d_ghosts<T, 4>(a, g, x, yy, own, nbW, nbE, nbS, nbN);
+        float f[MLP_IN];
+        crk::mlp_features<T, NM>(c, nbE, nbW, nbN, nbS, a.mlp_scale, f);
+#pragma unroll
+        for (int k = 0; k < MLP_IN; ++k) out[threadIdx.x * (MLP_IN + 1) + k] = f[k];
+        T gam;
+        if constexpr (sizeof(T) == 4) gam = a.gammaf;
+        else gam = a.gamma;
+        const bool fl = crk::tvb_limit_cell<T, 4, NM>(c, nbW, nbE, nbS, nbN, T(g.Mdx2), T(g.Mdy2), gam);
+        y[(size_t)yy * nx + x] = fl ? 1.f : 0.f;
     }
-    float f[MLP_IN];
-    crk::mlp_features<T, NM>(c, nb[1], nb[0], nb[3], nb[2], Mh2, f);
-    const size_t cell = (size_t)yy * nx + x;
-    for (int k = 0; k < MLP_IN; ++k) X[cell * MLP_IN + k] = f[k];
-    const bool fl = crk::tvb_limit_cell<T, 4, NM>(c, nb[0], nb[1], nb[2], nb[3], T(a.M * a.dx * a.dx),
-                                                  T(a.M * a.dy * a.dy), T(a.gamma));
-    y[cell] = fl ? 1.f : 0.f;
+    __syncthreads();
+    const int cells = min(FEAT_THREADS, nx - x0);
+    float* Xb = X + ((size_t)yy * nx + x0) * MLP_IN;
+    for (int i = threadIdx.x; i < cells * MLP_IN; i += FEAT_THREADS) Xb[i] = out[i / MLP_IN * (MLP_IN + 1) + i % MLP_IN];
 }
 
 uint64_t splitmix(uint64_t& s) {
@@ -544,9 +583,24 @@ int crkdg_mlp_train(crkdg_mlp* m, const float* X_dev, const float* y_dev, int n,
 
 int crkdg_mlp_predict(crkdg_mlp* m, const float* X_dev, int n, float* logits_dev) {
     if (!m || !X_dev || !logits_dev || n < 1) return mfail(CRKDG_EINVAL, "bad argument");
-    const size_t smem = sizeof(crk::MlpSmem) + 4 * (32 * crk::MLP_INP + 64) * sizeof(__nv_bfloat16);
-    cudaFuncSetAttribute(mlp_predict_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    mlp_predict_kernel<<<(n + 127) / 128, 128, smem, m->stream>>>(m->d_prm, X_dev, n, logits_dev);
+    const size_t smem =
+        sizeof(crk::MlpSmem) + (PREDICT_THREADS / 32) * (32 * crk::MLP_INP + 64) * sizeof(__nv_bfloat16);
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    static int per_sm = 1;
+    std::call_once(once, [&] {
+        for (auto k : {mlp_predict_kernel<true>, mlp_predict_kernel<false>})
+            if (attr_err == cudaSuccess)
+                attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (attr_err == cudaSuccess)
+            attr_err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_predict_kernel<true>,
+                                                                     PREDICT_THREADS, smem);
+    });
+    MCK(attr_err);
+    const long long tiles = ((long long)n + PREDICT_THREADS - 1) / PREDICT_THREADS;
+    const int grid = (int)std::min<long long>(tiles, (long long)std::max(1, per_sm) * std::max(1, crk::sm_count()));
+    auto kern = reinterpret_cast<uintptr_t>(X_dev) % 8 == 0 ? mlp_predict_kernel<true> : mlp_predict_kernel<false>;
+    kern<<<grid, PREDICT_THREADS, smem, m->stream>>>(m->d_prm, X_dev, n, logits_dev);
     MCK(cudaGetLastError());
     MCK(cudaStreamSynchronize(m->stream));
     return CRKDG_OK;
@@ -574,18 +628,16 @@ int crkdg_mlp_predict_tc(crkdg_mlp* m, const float* X_dev, int n, float* logits_
 int crkdg_features_impl(const StepArgs& a, int precision, int k, int basis, const void* u, float* X, float* y,
                         double Mh2, cudaStream_t st) {
     if (k != 2) return mfail(CRKDG_EUNSUPPORTED, "the learned indicator is built for k = 2");
-    dim3 grid((a.nx + 127) / 128, a.ny);
-    if (precision == CRKDG_F64) {
-        if (basis == CRKDG_BASIS_P)
-            features_kernel<double, 2, 0><<<grid, 128, 0, st>>>(a, (const double*)u, X, y, Mh2);
-        else
-            features_kernel<double, 2, 1><<<grid, 128, 0, st>>>(a, (const double*)u, X, y, Mh2);
-    } else {
-        if (basis == CRKDG_BASIS_P)
-            features_kernel<float, 2, 0><<<grid, 128, 0, st>>>(a, (const float*)u, X, y, Mh2);
-        else
-            features_kernel<float, 2, 1><<<grid, 128, 0, st>>>(a, (const float*)u, X, y, Mh2);
-    }
+    StepArgs b = a;
+    crk::set_derived(b);
+    b.mlp_scale = (float)Mh2;
+    const dim3 grid((a.nx + FEAT_THREADS - 1) / FEAT_THREADS, a.ny);
+    auto run = [&](auto kern, auto* state) { kern<<<grid, FEAT_THREADS, 0, st>>>(b, state, X, y); };
+    const bool P = basis == CRKDG_BASIS_P;
+    if (precision == CRKDG_F64)
+        run(P ? features_kernel<double, 2, 0> : features_kernel<double, 2, 1>, (const double*)u);
+    else
+        run(P ? features_kernel<float, 2, 0> : features_kernel<float, 2, 1>, (const float*)u);
     MCK(cudaGetLastError());
     return CRKDG_OK;
 }

@@ -13,7 +13,10 @@ namespace crk {
 constexpr int MLP_IN = 40, MLP_INP = 48, MLP_H = 64;
 constexpr int MLP_NPARAM = MLP_H * MLP_IN + MLP_H + 2 * (MLP_H * MLP_H + MLP_H) + MLP_H + 1;   // 11009
 
-// Weights as the tensor cores read them (B operands are W rows: k contiguous)
+// Weights as the tensor cores read them (B operands are W rows: k contiguous;
+// in the 64-wide rows the 8-value groups of row r are permuted by r % 8, see
+// mlp_swz: a fragment's 8 rows lie 128 bytes apart, and unpermuted all in the
+// same four banks)
 struct MlpSmem {
     __nv_bfloat16 W1[MLP_H * MLP_INP];   // layer 1, input padded 40 -> 48 with zeros
     __nv_bfloat16 W2[MLP_H * MLP_H];
@@ -21,6 +24,9 @@ struct MlpSmem {
     __nv_bfloat16 W4[8 * MLP_H];         // output row 0, rows 1..7 zero
     float b1[MLP_H], b2[MLP_H], b3[MLP_H], b4[8];
 };
+
+// position of element k in row r of a 64-wide weight matrix
+__host__ __device__ constexpr int mlp_swz(int r, int k) { return k ^ ((r & 7) << 3); }
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -44,7 +50,7 @@ __device__ __forceinline__ void c_to_a(const float (&c0)[4], const float (&c1)[4
 }
 
 // One hidden layer: acc[nt] = bias + A * W^T over KS k-slices of 16
-template <int KS>
+template <int KS, bool SWZ>
 __device__ __forceinline__ void mlp_layer(const uint32_t (&a)[KS][4], const __nv_bfloat16* W, const float* bias,
                                           int ldw, float (&acc)[8][4], int g, int tig) {
 #pragma unroll
@@ -57,23 +63,20 @@ __device__ __forceinline__ void mlp_layer(const uint32_t (&a)[KS][4], const __nv
         const __nv_bfloat16* wr = W + (size_t)(nt * 8 + g) * ldw;
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
-            const uint32_t bb0 = *reinterpret_cast<const uint32_t*>(wr + ks * 16 + 2 * tig);
-            const uint32_t bb1 = *reinterpret_cast<const uint32_t*>(wr + ks * 16 + 8 + 2 * tig);
+            const int k0 = SWZ ? mlp_swz(g, ks * 16) : ks * 16, k1 = SWZ ? mlp_swz(g, ks * 16 + 8) : ks * 16 + 8;
+            const uint32_t bb0 = *reinterpret_cast<const uint32_t*>(wr + k0 + 2 * tig);
+            const uint32_t bb1 = *reinterpret_cast<const uint32_t*>(wr + k1 + 2 * tig);
             mma_bf16(acc[nt], a[ks], bb0, bb1);
         }
     }
 }
 
-// Logits of the 32 cells held by the warp's lanes.  feat: this lane's 40
-// features; stage: the warp's 32 x 48 BF16 staging area (+ 32 floats after it).
-__device__ __forceinline__ float mlp_warp_logit(const MlpSmem& w, const float* feat, __nv_bfloat16* stage) {
+// Logits of the 32 cells whose features fill the warp's 32 x 48 BF16 staging
+// area (+ 32 floats after it); lane l returns cell l's.
+__device__ __forceinline__ float mlp_warp_staged(const MlpSmem& w, __nv_bfloat16* stage) {
     const int lane = threadIdx.x & 31;
     const int g = lane >> 2, tig = lane & 3;
     float* lout = reinterpret_cast<float*>(stage + 32 * MLP_INP);
-#pragma unroll
-    for (int f = 0; f < MLP_INP; f += 2)
-        *reinterpret_cast<uint32_t*>(stage + lane * MLP_INP + f) =
-            pack_bf16(f < MLP_IN ? feat[f] : 0.f, f + 1 < MLP_IN ? feat[f + 1] : 0.f);
     __syncwarp();
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
@@ -89,13 +92,13 @@ __device__ __forceinline__ float mlp_warp_logit(const MlpSmem& w, const float* f
         }
         float acc[8][4];
         uint32_t ah[4][4];
-        mlp_layer<3>(a1, w.W1, w.b1, MLP_INP, acc, g, tig);
+        mlp_layer<3, false>(a1, w.W1, w.b1, MLP_INP, acc, g, tig);
 #pragma unroll
         for (int t = 0; t < 4; ++t) c_to_a(acc[2 * t], acc[2 * t + 1], ah[t]);
-        mlp_layer<4>(ah, w.W2, w.b2, MLP_H, acc, g, tig);
+        mlp_layer<4, true>(ah, w.W2, w.b2, MLP_H, acc, g, tig);
 #pragma unroll
         for (int t = 0; t < 4; ++t) c_to_a(acc[2 * t], acc[2 * t + 1], ah[t]);
-        mlp_layer<4>(ah, w.W3, w.b3, MLP_H, acc, g, tig);
+        mlp_layer<4, true>(ah, w.W3, w.b3, MLP_H, acc, g, tig);
 #pragma unroll
         for (int t = 0; t < 4; ++t) c_to_a(acc[2 * t], acc[2 * t + 1], ah[t]);
         // output layer: one 8-column tile, column 0 is the logit
@@ -103,8 +106,8 @@ __device__ __forceinline__ float mlp_warp_logit(const MlpSmem& w, const float* f
         const __nv_bfloat16* wr = w.W4 + (size_t)g * MLP_H;
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
-            const uint32_t bb0 = *reinterpret_cast<const uint32_t*>(wr + ks * 16 + 2 * tig);
-            const uint32_t bb1 = *reinterpret_cast<const uint32_t*>(wr + ks * 16 + 8 + 2 * tig);
+            const uint32_t bb0 = *reinterpret_cast<const uint32_t*>(wr + mlp_swz(g, ks * 16) + 2 * tig);
+            const uint32_t bb1 = *reinterpret_cast<const uint32_t*>(wr + mlp_swz(g, ks * 16 + 8) + 2 * tig);
             mma_bf16(o, ah[ks], bb0, bb1);
         }
         if (tig == 0) {
@@ -116,6 +119,16 @@ __device__ __forceinline__ float mlp_warp_logit(const MlpSmem& w, const float* f
     const float z = lout[lane];
     __syncwarp();
     return z;
+}
+
+// The same from each lane's 40 features
+__device__ __forceinline__ float mlp_warp_logit(const MlpSmem& w, const float* feat, __nv_bfloat16* stage) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int f = 0; f < MLP_INP; f += 2)
+        *reinterpret_cast<uint32_t*>(stage + lane * MLP_INP + f) =
+            pack_bf16(f < MLP_IN ? feat[f] : 0.f, f + 1 < MLP_IN ? feat[f + 1] : 0.f);
+    return mlp_warp_staged(w, stage);
 }
 
 // Load the BF16 weights and FP32 biases of a packed parameter vector (device,
@@ -135,10 +148,12 @@ __device__ __forceinline__ void mlp_load_smem(MlpSmem& w, const float* __restric
         w.W1[i] = __float2bfloat16_rn(c < MLP_IN ? W1[r * MLP_IN + c] : 0.f);
     }
     for (int i = threadIdx.x; i < MLP_H * MLP_H; i += blockDim.x) {
-        w.W2[i] = __float2bfloat16_rn(W2[i]);
-        w.W3[i] = __float2bfloat16_rn(W3[i]);
+        const int r = i / MLP_H, o = r * MLP_H + mlp_swz(r, i % MLP_H);
+        w.W2[o] = __float2bfloat16_rn(W2[i]);
+        w.W3[o] = __float2bfloat16_rn(W3[i]);
     }
-    for (int i = threadIdx.x; i < 8 * MLP_H; i += blockDim.x) w.W4[i] = __float2bfloat16_rn(i < MLP_H ? W4[i] : 0.f);
+    for (int i = threadIdx.x; i < 8 * MLP_H; i += blockDim.x)   // row 0: not permuted; the others are zero
+        w.W4[i] = __float2bfloat16_rn(i < MLP_H ? W4[i] : 0.f);
     for (int i = threadIdx.x; i < MLP_H; i += blockDim.x) {
         w.b1[i] = b1[i];
         w.b2[i] = b2[i];
