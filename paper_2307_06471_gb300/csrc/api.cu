@@ -282,6 +282,29 @@ int linear_shape(crkdg_ctx* c) {
     return CRKDG_OK;
 }
 
+// constants of the modal step: gamma_l = b^T A^l 1 of the tableau (FP64, host)
+// and the inflow faces
+void set_linear(const crkdg_ctx* c, StepArgs& a) {
+    const int s = c->tab.s;
+    double v[crk::MAXS];
+    for (int i = 0; i < s; ++i) v[i] = 1.0;
+    for (int l = 0; l < crk::MAXS; ++l) {
+        double g = 0.0;
+        if (l < s)
+            for (int i = 0; i < s; ++i) g += c->tab.b[i] * v[i];
+        a.lin_gamma[l] = g;
+        a.lin_gammaf[l] = (float)g;
+        double nv[crk::MAXS];
+        for (int i = 0; i < s; ++i) {
+            nv[i] = 0.0;
+            for (int j = 0; j < s; ++j) nv[i] += c->tab.a[i * CRKDG_MAX_STAGES + j] * v[j];
+        }
+        for (int i = 0; i < s; ++i) v[i] = nv[i];
+    }
+    a.lin_inflow = (a.beta[0] > 0.0 ? 1 : 0) | (a.beta[0] < 0.0 ? 2 : 0) | (a.beta[1] > 0.0 ? 4 : 0) |
+                   (a.beta[1] < 0.0 ? 8 : 0);
+}
+
 // the pending limit as an in-place pass over u[cur]; troubled cells are
 // counted into the run state, where the next step's epilogue reports them
 int enqueue_limit_pass(crkdg_ctx* c, double M, int dt_from_dev) {
@@ -361,25 +384,7 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
                 r = ensure_partials(c, (size_t)lns * lnseg * 8);
                 if (r) return r;
                 a.partials = c->d_partials;
-                // gamma_l = b^T A^l 1 of the tableau (FP64, host)
-                const int s = c->tab.s;
-                double v[crk::MAXS];
-                for (int i = 0; i < s; ++i) v[i] = 1.0;
-                for (int l = 0; l < crk::MAXS; ++l) {
-                    double g = 0.0;
-                    if (l < s)
-                        for (int i = 0; i < s; ++i) g += c->tab.b[i] * v[i];
-                    a.lin_gamma[l] = g;
-                    a.lin_gammaf[l] = (float)g;
-                    double nv[crk::MAXS];
-                    for (int i = 0; i < s; ++i) {
-                        nv[i] = 0.0;
-                        for (int j = 0; j < s; ++j) nv[i] += c->tab.a[i * CRKDG_MAX_STAGES + j] * v[j];
-                    }
-                    for (int i = 0; i < s; ++i) v[i] = nv[i];
-                }
-                a.lin_inflow = (a.beta[0] > 0.0 ? 1 : 0) | (a.beta[0] < 0.0 ? 2 : 0) | (a.beta[1] > 0.0 ? 4 : 0) |
-                               (a.beta[1] < 0.0 ? 8 : 0);
+                set_linear(c, a);
                 CK(crk::launch_step2d_linear(c->precision, c->k, c->basis, a, c->lin_wpb, c->stream));
             } else {
                 CK(crk::launch_step2d(c->kphys, c->precision, c->k, c->basis, a, c->wpb, c->stream));
@@ -388,6 +393,7 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
     } else {
         const int warps = (c->mesh.nx + 29) / 30;
         const int blocks = (warps + 7) / 8;
+        set_linear(c, a);
         CK(crk::launch_step1d(c->kphys, c->precision, c->k, a, 1, blocks == 1 ? warps * 32 : 256, blocks, c->stream));
     }
     c->cur ^= 1;
@@ -916,14 +922,19 @@ int crkdg_run_fixed(crkdg_ctx* c, int n_steps, double dt) {
         }
         return CRKDG_OK;
     }
-    // whole run in one single-block launch
+    // whole run in one launch of one cluster
     if (n_steps == 0) return CRKDG_OK;
     StepArgs a = base_args(c);
     a.uin = c->u[c->cur];
     a.uout = c->u[c->cur ^ 1];
     a.t = c->t;
     a.dt = dt;
-    CK(crk::launch_step1d(c->kphys, c->precision, c->k, a, n_steps, warps * 32, 1, c->stream));
+    set_linear(c, a);
+    // a power of two of blocks, up to 8, for a warp each where that reaches
+    int blocks = 1;
+    while (blocks < 8 && blocks < warps) blocks *= 2;
+    CK(crk::launch_step1d(c->kphys, c->precision, c->k, a, n_steps, (warps + blocks - 1) / blocks * 32, blocks,
+                          c->stream));
     if (n_steps % 2) c->cur ^= 1;
     c->t += n_steps * dt;
     return CRKDG_OK;

@@ -16,14 +16,32 @@ cudaError_t run_step1d(const StepArgs& a, int n_steps, int threads, int blocks, 
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaFuncAttributes fa;   // what its static shared memory leaves of a block's 227 KB
+        attr_err = cudaFuncGetAttributes(&fa, kern);
+        if (attr_err == cudaSuccess)
+            attr_err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            227 * 1024 - (int)fa.sharedSizeBytes);
     });
     if (attr_err != cudaSuccess) return attr_err;
     const size_t smem = (size_t)(a.s > 1 ? a.s - 1 : 1) * NDOF * sizeof(T) * threads;
     StepArgs b = a;
     set_derived(b);
-    kern<<<blocks, threads, smem, st>>>(b, n_steps);
-    return cudaGetLastError();
+    if (n_steps == 1) {
+        kern<<<blocks, threads, smem, st>>>(b, n_steps);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};   // a run: one cluster
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = blocks;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, b, n_steps);
 }
 
 template <class T, int K, int PHYS>
