@@ -299,8 +299,8 @@ int crkdg_get_limit_mode(const crkdg_ctx* ctx, int* mode);
 
 /* How the 2D step evaluates its operators for linear advection.
  * CRKDG_FORM_AUTO (default): where the flux is linear (CRKDG_ADVECTION, FP32
- * or FP64) and every non-periodic side is outflow, wall or a constant state,
- * the step uses the modal form of the operators — the local operator (eq.
+ * or FP64) and every non-periodic side is outflow, wall, a constant state or
+ * sine data (CRKDG_FN_SINE, CRKDG_FN_SINE_PROD), the step uses the modal form of the operators — the local operator (eq.
  * (2.7)) is beta . grad of the modal polynomial, the final stage's
  * sum_i b_i div^DG f(u^(i)) equals the DG operator of sum_i b_i u^(i) (the
  * linearity behind Theorem 3.3), applied once with the upwind flux — which

@@ -85,6 +85,7 @@ struct crkdg_ctx {
     double* d_stage = nullptr;            // FP64 staging of state I/O for FP32 states (first use)
     int op_form = CRKDG_FORM_AUTO;        // crkdg_set_operator_form
     int lin_seg_rows = 0, lin_wpb = 0;    // launch shape of the modal linear step (first use)
+    void* d_lin_data = nullptr;           // its boundary data
     bool owns_state = true;               // false: u[0], u[1] are the caller's (crkdg_create_on_buffers)
     std::map<GraphKey, cudaGraphExec_t> graphs;
 };
@@ -245,7 +246,7 @@ int enqueue_reduce(crkdg_ctx* c, crk::ReduceRun run) {
 }
 
 // the modal step applies: linear flux, 2D, FP32/FP64, every non-periodic side
-// affine (outflow, wall, constant state), not switched off
+// affine (outflow, wall, constant state) or sine data, not switched off
 bool use_linear(const crkdg_ctx* c) {
     if (c->op_form != CRKDG_FORM_AUTO || c->kphys != crk::PHYS_ADV || c->dim != 2 ||
         compensated(c->precision))
@@ -258,7 +259,9 @@ bool use_linear(const crkdg_ctx* c) {
     }
     crk::set_bc_affine(bc, 1);
     for (int s = 0; s < 4; ++s)
-        if (bc[s].type != crk::BC_PERIODIC && !bc[s].affine) return false;
+        if (bc[s].type != crk::BC_PERIODIC && !bc[s].affine &&
+            !(bc[s].type == crk::BC_DIRICHLET && (bc[s].fn == crk::FN_SINE || bc[s].fn == crk::FN_SINE_PROD)))
+            return false;
     return true;
 }
 
@@ -266,8 +269,15 @@ bool use_linear(const crkdg_ctx* c) {
 // memory let the device's SMs hold, segments of >= 1 row
 int linear_shape(crkdg_ctx* c) {
     if (c->lin_seg_rows > 0) return CRKDG_OK;
+    // the boundary faces' data
+    const size_t data = (size_t)2 * (c->mesh.nx + c->mesh.ny) * (c->k + 1) * c->esize;
+    if (!c->d_lin_data && cudaMalloc(&c->d_lin_data, data) != cudaSuccess) {
+        cudaGetLastError();
+        c->d_lin_data = nullptr;
+        return fail(CRKDG_ENOMEM, "cudaMalloc of the boundary data failed");
+    }
     crk::KernelInfo ki;
-    CK(crk::info_step2d_linear(c->precision, c->k, c->basis, c->tab.s, &ki));
+    CK(crk::info_step2d_linear(c->precision, c->k, c->basis, &ki));
     const int wpb = std::max(1, std::min(4, ki.max_threads / 32));
     const int regs_warp = ((ki.regs + 7) / 8) * 8 * 32;
     const int by_regs = 65536 / regs_warp;
@@ -279,6 +289,9 @@ int linear_shape(crkdg_ctx* c) {
     const int L = (int)std::max(1L, ((long)c->mesh.ny + nseg - 1) / nseg);
     c->lin_seg_rows = std::min(L, c->mesh.ny);
     c->lin_wpb = wpb;
+    // few warps: blocks small enough to reach every SM
+    const long warps = (long)ns * ((c->mesh.ny + c->lin_seg_rows - 1) / c->lin_seg_rows);
+    while (c->lin_wpb > 1 && warps < (long)c->lin_wpb * crk::sm_count()) c->lin_wpb /= 2;
     return CRKDG_OK;
 }
 
@@ -384,6 +397,7 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
                 r = ensure_partials(c, (size_t)lns * lnseg * 8);
                 if (r) return r;
                 a.partials = c->d_partials;
+                a.lin_data = c->d_lin_data;
                 set_linear(c, a);
                 CK(crk::launch_step2d_linear(c->precision, c->k, c->basis, a, c->lin_wpb, c->stream));
             } else {
@@ -525,6 +539,9 @@ int create_impl(const crkdg_mesh* mesh, int k, int basis, int flux, const crkdg_
     if (c->dim == 2 && !use_linear(c)) {   // a step allocates nothing
         r = ensure_step_scratch(c);
         if (r) return bail(r);
+    } else if (c->dim == 2) {
+        r = linear_shape(c);
+        if (r) return bail(r);
     }
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return bail(fail(CRKDG_ECUDA, "stream sync failed"));
     *out = c;
@@ -602,6 +619,7 @@ void crkdg_destroy(crkdg_ctx* c) {
     if (c->d_state) cudaFree(c->d_state);
     if (c->d_partials) cudaFree(c->d_partials);
     if (c->d_seam) cudaFree(c->d_seam);
+    if (c->d_lin_data) cudaFree(c->d_lin_data);
     if (c->d_flags) cudaFree(c->d_flags);
     if (c->u3) cudaFree(c->u3);
     if (c->d_stage) cudaFree(c->d_stage);

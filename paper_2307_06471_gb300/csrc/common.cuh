@@ -93,6 +93,9 @@ struct StepArgs {
     // operator D: lin_gamma[l] = b^T A^l 1 (the modal linear step)
     double lin_gamma[MAXS];
     float lin_gammaf[MAXS];
+    // modal step: trace coefficients of sum_i b_i of the sine boundary data at the
+    // stage times, per boundary face, sides W, E (ny faces), S, N (nx) in turn
+    void* lin_data;
     int lin_inflow;           // inflow faces of every cell: bit 0 W, 1 E, 2 S, 3 N (the modal linear step)
     // limiter parameters as the one-thread-per-cell limiter pass takes them
     // (filled by set_limiter_params at its launch)
@@ -314,15 +317,6 @@ __device__ __forceinline__ void llf_ax(const Phys<T, PHYS>& ph, const T* uL, con
 template <int AXIS, bool HALF = true, class T>
 __device__ __forceinline__ void llf_ax(const EulerDev<T>& ph, const T* uL, const T* uR, T* F) {
     llf<T, AXIS, HALF>(ph, uL, uR, F);
-}
-
-// The Lax--Friedrichs flux of llf from states whose normal fluxes and wave
-// speeds are already known (the same arithmetic as llf).
-template <class T, int NV>
-__device__ __forceinline__ void lf_from_fluxes(const T* uL, const T* fL, T sL, const T* uR, const T* fR, T sR, T* F) {
-    const T al = sL > sR ? sL : sR;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = T(0.5) * ((fL[v] + fR[v]) - al * (uR[v] - uL[v]));
 }
 
 // Value of the sine boundary data (FN_SINE, FN_SINE_PROD); kept out of line

@@ -19,8 +19,14 @@
 // The work decomposition is step2d.cuh's (marching warps, 30 columns + 2 halo
 // lanes, segments of rows, the row below finished when the current row's
 // south trace is known) with a tenth of its arithmetic, so the step is bound
-// by HBM.  Boundary sides: periodic, or an exterior state affine in the
-// interior one (outflow, wall, constant state; BCSide::affine).
+// by HBM.  Boundary sides: periodic, an exterior state affine in the
+// interior one (outflow, wall, constant state; BCSide::affine), or sine data,
+// whose part of the final stage's flux is the projection of sum_i b_i g(., t^n +
+// c_i dt) onto the face's Legendre polynomials by the face rule: formed for all
+// boundary faces by boundary_traces_kernel, one thread per (face, point, stage).
+// (The quadrature step evaluates the data in the boundary warps, a stage and
+// point after another, each an FP64 sine on the narrow FP64 pipe: with it Q^3
+// RK4 in FP64 on 80 x 80 cells took 1.38 ms a step; the two launches of this form take 0.034.)
 #pragma once
 #include "step2d.cuh"
 
@@ -57,13 +63,60 @@ constexpr double lin_deta(int r, int c) {
     return (ic == ir && jc > jr && (jc - jr) % 2 == 1) ? 2.0 * jr + 1.0 : 0.0;
 }
 
-// private shared memory per thread (none: the stages are combined in registers)
-template <class T, int K, int B>
-__host__ __device__ constexpr int linear_smem_per_thread(int) {
-    return 0;
+// a side whose exterior state is sine data
+__host__ __device__ inline bool lin_data_side(const BCSide& b) {
+    return b.type == BC_DIRICHLET && (b.fn == FN_SINE || b.fn == FN_SINE_PROD);
+}
+__host__ __device__ inline size_t lin_data_offset(int side, int nx, int ny, int nq) {
+    return (size_t)nq * (side == 0 ? 0 : side == 1 ? ny : side == 2 ? 2 * (size_t)ny : 2 * (size_t)ny + nx);
 }
 
-template <class T, int K, int B>
+constexpr int BT_FACES = 2;   // faces per block
+template <class T, int K>
+__global__ void __launch_bounds__(BT_FACES * (K + 1) * MAXS) boundary_traces_kernel(const StepArgs a) {
+    constexpr int NQ = K + 1;
+    __shared__ T g[BT_FACES][NQ][MAXS];
+    allow_dependent_launch();
+    const int side = blockIdx.y, S = a.s;
+    const BCSide& bc = a.bc[side];
+    if (!lin_data_side(bc)) return;
+    const double t0 = a.dt_from_dev ? a.ds->t : a.t, dt = a.dt_from_dev ? a.ds->dt : a.dt;
+    if (!(dt > 0.0)) return;
+    const int i = threadIdx.x % S, p = threadIdx.x / S % NQ, f = threadIdx.x / (S * NQ);
+    const int face = blockIdx.x * BT_FACES + f;
+    const bool valid = face < (side < 2 ? a.ny : a.nx);
+    if (valid) {
+        double xi = 0.0;
+        static_for<NQ>([&](auto q) {
+            if (q == p) xi = make_tab1d<K>().xq[decltype(q)::value];
+        });
+        const double x = side == 0 ? a.x0 : side == 1 ? a.x0 + a.nx * a.dx : a.x0 + (face + 0.5) * a.dx + 0.5 * a.dx * xi;
+        const double y = side == 2 ? a.y0 : side == 3 ? a.y0 + a.ny * a.dy : a.y0 + (face + 0.5 + 0.5 * xi) * a.dy;
+        const T bi = tab_bT<T>(a, i);
+        g[f][p][i] = bi == T(0) ? T(0)
+                                : bi * T(bc_sine_value(bc.fn == FN_SINE_PROD, bc.p[0], bc.p[1], bc.p[2], bc.p[3], bc.p[4],
+                                                       x, y, t0 + tab_c(a, i) * dt));
+    }
+    __syncthreads();
+    if (!valid || i != 0) return;
+    T* out = static_cast<T*>(a.lin_data) + lin_data_offset(side, a.nx, a.ny, NQ) + (size_t)face * NQ;
+    T e = T(0);   // the coefficient of P_p
+    static_for<NQ>([&](auto pp) {
+        T gp = T(0);
+        for (int j = 0; j < S; ++j) gp += g[f][pp][j];
+        static_for<NQ>([&](auto q) {
+            constexpr double w = make_tab1d<K>().pw[decltype(pp)::value][decltype(q)::value];
+            if (q == p) e = fma(gp, T(w), e);
+        });
+    });
+    out[p] = e;
+}
+
+// DATA: some side has sine data.  TRIM: one halo row at most, of which only the
+// traces are formed (FP64, whose pipe is the bound, and DATA; for the plain FP32
+// step, bound by the latency of its loads, the branches cost more than the
+// rows: 0.320 against 0.270 ms on 4096^2 Q^2 cells).
+template <class T, int K, int B, bool DATA>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d_linear_kernel(const StepArgs a) {
     constexpr int NM = n_modes_2d(K, B);
     constexpr int NT = K + 1;   // trace coefficients per face
@@ -71,6 +124,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
     const int tid = threadIdx.x;
     const int lane = tid & 31;
 
+    constexpr bool TRIM = DATA || sizeof(T) == 8;
+    if constexpr (DATA) wait_for_step();   // for the boundary data
     allow_dependent_launch();
     const int gw = blockIdx.x * (nthr >> 5) + (tid >> 5);
     const int total_warps = a.n_strips * a.n_segs;
@@ -94,8 +149,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
     const bool outlane = lane >= 1 && lane <= 30 && col < nx;
     const int r0 = (int)(((long long)seg * ny) / a.n_segs);
     const int r1 = (int)(((long long)(seg + 1) * ny) / a.n_segs);
-    const int rstart = (r0 > 0 || pery) ? r0 - 1 : r0;
-    const int rend = (r1 < ny || pery) ? r1 : r1 - 1;
+    // the row below is needed for its north trace where the south faces are
+    // inflow faces, the row above likewise: one halo row at most
+    const int rstart = (!TRIM || (a.lin_inflow & 4)) && (r0 > 0 || pery) ? r0 - 1 : r0;
+    const int rend = (!TRIM || (a.lin_inflow & 8)) && (r1 < ny || pery) ? r1 : r1 - 1;
 
     if (!(dt > 0.0)) {   // a non-positive dt leaves the state unchanged
         if (outlane)
@@ -130,9 +187,16 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
             out[m] = acc;
         });
     };
-    // exterior trace at a non-periodic side: m * interior + constant state
-    auto bc_trace = [&](int side, const T* in, T* out) {
+    // exterior trace at a non-periodic side: m * interior + constant state, or
+    // the side's data at its face `face`
+    auto bc_trace = [&](int side, int face, const T* in, T* out) {
         const BCSide& b = a.bc[side];
+        if (DATA && !b.affine) {
+            const T* d = static_cast<const T*>(a.lin_data) + lin_data_offset(side, nx, ny, NT) + (size_t)face * NT;
+#pragma unroll
+            for (int q = 0; q < NT; ++q) out[q] = d[q];
+            return;
+        }
         const T c = sizeof(T) == 4 ? T(b.cf[0]) : T(b.cd[0]);
 #pragma unroll
         for (int q = 0; q < NT; ++q) out[q] = T(b.m[0]) * in[q] + (q == 0 ? c : T(0));
@@ -206,8 +270,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
         }
 
         // DG operator of wbar: local part, then the inflow-face jumps
-        T Lw[NM];
-        applyD(wbar, Lw);
+        T Lw[NM];   // (of a halo row only the traces are used)
+        if (!TRIM || out_row) applyD(wbar, Lw);
         T tE[NT], tW[NT], tN[NT], tS[NT];
 #pragma unroll
         for (int q = 0; q < NT; ++q) tE[q] = tW[q] = tN[q] = tS[q] = T(0);
@@ -227,9 +291,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
             extW[q] = shfl_up(tE[q], 1);     // west neighbour's east trace
             extE[q] = shfl_down(tW[q], 1);   // east neighbour's west trace
         }
-        if (!perx && col == 0) bc_trace(0, tW, extW);
-        if (!perx && col == nx - 1) bc_trace(1, tE, extE);
-        if (inW) {
+        const int ry = r < 0 ? r + ny : (r >= ny ? r - ny : r);
+        if ((!DATA || inW) && !perx && col == 0) bc_trace(0, ry, tW, extW);
+        if ((!DATA || inE) && !perx && col == nx - 1) bc_trace(1, ry, tE, extE);
+        if (inW && (!TRIM || out_row)) {
             static_for<NM>([&](auto mc) {
                 constexpr int m = decltype(mc)::value;
                 constexpr int i = lin_mi<K, B>(m), j = lin_mj<K, B>(m);
@@ -237,17 +302,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
                 Lw[m] += (kW * T(f)) * (extW[j] - tW[j]);
             });
         }
-        if (inE) {
+        if (inE && (!TRIM || out_row)) {
             static_for<NM>([&](auto mc) {
                 constexpr int m = decltype(mc)::value;
                 constexpr int i = lin_mi<K, B>(m), j = lin_mj<K, B>(m);
                 Lw[m] += (kE * T(2.0 * i + 1.0)) * (extE[j] - tE[j]);
             });
         }
-        if (inS && (r > rstart || south_bc)) {
+        if (inS && (!TRIM || out_row) && (r > rstart || south_bc)) {
             T extS[NT];
-            if (south_bc) {
-                bc_trace(2, tS, extS);
+            if (south_bc) {   // lanes past the east side read nothing of theirs
+                if (!DATA || outlane) bc_trace(2, col, tS, extS);
             } else {
 #pragma unroll
                 for (int q = 0; q < NT; ++q) extS[q] = prevN[q];
@@ -261,7 +326,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
         }
 
         // the row below: its north face is this row's south face
-        if (r > rstart && r - 1 >= r0 && r - 1 < r1) {
+        if (TRIM ? r > r0 && r - 1 < r1 : r > rstart && r - 1 >= r0 && r - 1 < r1) {
             if (inN) {
                 static_for<NM>([&](auto mc) {
                     constexpr int m = decltype(mc)::value;
@@ -277,13 +342,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
             if (r == ny - 1 && !pery) {   // top boundary: north face from the boundary state
                 if (inN) {
                     T extN[NT];
-                    bc_trace(3, tN, extN);
+                    if (!DATA || outlane) bc_trace(3, col, tN, extN);
                     static_for<NM>([&](auto mc) {
                         constexpr int m = decltype(mc)::value;
                         constexpr int i = lin_mi<K, B>(m), j = lin_mj<K, B>(m);
                         P[m] -= tdt * ((kN * T(2.0 * j + 1.0)) * (extN[i] - tN[i]));
                     });
                 }
+                write_row(r);
+            } else if (TRIM && r == rend) {   // outflow through the north faces
                 write_row(r);
             }
         }
