@@ -64,8 +64,7 @@ struct TrainSmem {
 // of a thread's unit share its weights' 16-byte loads in the forward pass.
 // With tiles of 64 samples, a block per tile and unpadded rows (32-way bank
 // conflicts on the weights) a minibatch of 1024 took 0.126 ms; this takes
-// 0.023 ms (of which the weights' load and the chain of four layers there and
-// back are most: 8 warps an SM).
+// 0.014 ms (0.023 while the loads of the weights waited for one another).
 __global__ void __launch_bounds__(TRAIN_THREADS) mlp_fwdbwd_kernel(const float* __restrict__ prm,
                                                                    const float* __restrict__ X,
                                                                    const float* __restrict__ y,
@@ -75,10 +74,18 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_fwdbwd_kernel(const float* 
     extern __shared__ __align__(16) unsigned char sh_raw[];
     TrainSmem& sh = *reinterpret_cast<TrainSmem*>(sh_raw);
     const int tid = threadIdx.x, unit = tid & 63, sg = tid >> 6;   // unit of a layer, pair of samples
-    for (int i = tid; i < MLP_H * MLP_IN; i += TRAIN_THREADS) sh.W1[i / MLP_IN * SX + i % MLP_IN] = prm[OW1 + i];
-    for (int i = tid; i < MLP_H * MLP_H; i += TRAIN_THREADS) {
-        sh.W2[(i >> 6) * SH + (i & 63)] = prm[OW2 + i];
-        sh.W3[(i >> 6) * SH + (i & 63)] = prm[OW3 + i];
+    // (unrolled: the loads of a matrix are in flight together)
+    static_assert(MLP_H * MLP_IN % TRAIN_THREADS == 0 && MLP_H * MLP_H % TRAIN_THREADS == 0, "whole rounds");
+#pragma unroll
+    for (int r = 0; r < MLP_H * MLP_IN / TRAIN_THREADS; ++r) {
+        const int i = r * TRAIN_THREADS + tid;
+        sh.W1[i / MLP_IN * SX + i % MLP_IN] = __ldg(prm + OW1 + i);
+    }
+#pragma unroll
+    for (int r = 0; r < MLP_H * MLP_H / TRAIN_THREADS; ++r) {
+        const int i = r * TRAIN_THREADS + tid;
+        sh.W2[(i >> 6) * SH + (i & 63)] = __ldg(prm + OW2 + i);
+        sh.W3[(i >> 6) * SH + (i & 63)] = __ldg(prm + OW3 + i);
     }
     if (tid < MLP_H) {
         sh.b1[tid] = prm[OB1 + tid];
@@ -162,6 +169,7 @@ __global__ void __launch_bounds__(TRAIN_THREADS) mlp_fwdbwd_kernel(const float* 
         dense(sh.H2, MLP_H, SH, sh.W3, sh.b3, sh.H3);
         if (tid < TILE) {
             float z = sh.b4[0];
+#pragma unroll 16
             for (int k = 0; k < MLP_H; ++k) z = fmaf(sh.H3[tid * SH + k], sh.W4[k], z);
             float d = 0.f;
             if (tid < ns) {
@@ -229,7 +237,7 @@ __global__ void __launch_bounds__(REDUCE_RUNS * REDUCE_PARAMS)
     const int b0 = run * per, b1 = min(nblocks, b0 + per);
     float a = 0.f;
     if (p < MLP_NPARAM)
-#pragma unroll 8
+#pragma unroll 16
         for (int b = b0; b < b1; ++b) a += gpart[(size_t)b * MLP_NPARAM + p];
     part[run][t] = a;
     __syncthreads();
@@ -259,7 +267,7 @@ __global__ void __launch_bounds__(REDUCE_RUNS * REDUCE_PARAMS)
 // samples' features as one run of memory and rounds them into its staging area
 // (VEC: pairs, where X allows 8-byte loads).  A block per 128 samples that
 // loaded the weights each time, lanes reading 160 bytes apart and the weights'
-// rows in one bank group took 0.202 ms for 524,288 samples; this takes 0.057 ms.
+// rows in one bank group took 0.202 ms for 524,288 samples; this takes 0.055 ms.
 constexpr int PREDICT_THREADS = 128;
 template <bool VEC>
 __global__ void __launch_bounds__(PREDICT_THREADS) mlp_predict_kernel(const float* __restrict__ prm,

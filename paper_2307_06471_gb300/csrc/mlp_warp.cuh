@@ -143,10 +143,13 @@ __device__ __forceinline__ void mlp_load_smem(MlpSmem& w, const float* __restric
     const float* b3 = W3 + MLP_H * MLP_H;
     const float* W4 = b3 + MLP_H;
     const float* b4 = W4 + MLP_H;
+    // (unrolled: the loads of a matrix are in flight together)
+#pragma unroll 8
     for (int i = threadIdx.x; i < MLP_H * MLP_INP; i += blockDim.x) {
         const int r = i / MLP_INP, c = i % MLP_INP;
         w.W1[i] = __float2bfloat16_rn(c < MLP_IN ? W1[r * MLP_IN + c] : 0.f);
     }
+#pragma unroll 8
     for (int i = threadIdx.x; i < MLP_H * MLP_H; i += blockDim.x) {
         const int r = i / MLP_H, o = r * MLP_H + mlp_swz(r, i % MLP_H);
         w.W2[o] = __float2bfloat16_rn(W2[i]);
