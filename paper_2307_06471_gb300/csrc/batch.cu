@@ -105,6 +105,8 @@ struct crkdg_batch {
     unsigned* d_done = nullptr;
     double* d_partials = nullptr;
     double* d_tab = nullptr;
+    double* d_stage = nullptr;             // get_state's staging, as large as the largest problem read
+    size_t stage_cap = 0;
     unsigned long long* d_flags = nullptr;
     cudaStream_t stream = nullptr;
     int seg_rows = 32, wpb = 4;            // default_shape, crkdg_batch_set_launch
@@ -266,8 +268,8 @@ int start_run(crkdg_batch* b, double cfl, double t_end) {
 }
 
 int get_cur(const crkdg_batch* b, int p, int* cur) {
+    BCK(cudaMemcpyAsync(cur, b->d_curs + p, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     BCK(cudaStreamSynchronize(b->stream));
-    BCK(cudaMemcpy(cur, b->d_curs + p, sizeof(int), cudaMemcpyDeviceToHost));
     return CRKDG_OK;
 }
 
@@ -377,7 +379,7 @@ void crkdg_batch_destroy(crkdg_batch* b) {
     for (int i = 0; i < 2; ++i)
         if (b->buf[i]) cudaFree(b->buf[i]);
     for (void* p : {(void*)b->d_probs, (void*)b->d_tasks, (void*)b->d_flux, (void*)b->d_seams, b->d_seam, (void*)b->d_states, (void*)b->d_curs, (void*)b->d_done,
-                    (void*)b->d_partials, (void*)b->d_tab, (void*)b->d_flags, (void*)b->d_rows})
+                    (void*)b->d_partials, (void*)b->d_tab, (void*)b->d_stage, (void*)b->d_flags, (void*)b->d_rows})
         if (p) cudaFree(p);
     delete b;
 }
@@ -452,41 +454,41 @@ int crkdg_batch_get_state(crkdg_batch* b, int p, double* h) {
     if (r) return r;
     const BatchProblem& pb = b->probs[p];
     const size_t n = (size_t)pb.nx * pb.ny * b->nv * b->nm;
-    char* base = static_cast<char*>(b->buf[cur]) + pb.offset * b->esize;
+    const char* base = static_cast<char*>(b->buf[cur]) + pb.offset * b->esize;
+    const bool f32 = b->precision == CRKDG_F32;
+    // the copy a pending limiter is applied to, and the FP64 values of an FP32
+    // state: in the batch's staging buffer, kept between calls (FP64 first)
+    const size_t limited = b->pending ? (n * b->esize + 7) / 8 : 0, need = (f32 ? n : 0) + limited;
+    if (need > b->stage_cap) {
+        if (b->d_stage) cudaFree(b->d_stage);
+        b->d_stage = nullptr;
+        b->stage_cap = 0;
+        if (cudaMalloc(&b->d_stage, need * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            b->d_stage = nullptr;
+            return bfail(CRKDG_ENOMEM, "cudaMalloc failed");
+        }
+        b->stage_cap = need;
+    }
+    const void* src = base;
     if (b->pending) {
         // the stored state is pending the limiter of its last step: apply it to a copy
-        void* tmp = nullptr;
-        if (cudaMalloc(&tmp, n * b->esize) != cudaSuccess) return bfail(CRKDG_ENOMEM, "cudaMalloc failed");
-        cudaError_t e = cudaMemcpyAsync(tmp, base, n * b->esize, cudaMemcpyDeviceToDevice, b->stream);
+        void* tmp = b->d_stage + (f32 ? n : 0);
+        BCK(cudaMemcpyAsync(tmp, base, n * b->esize, cudaMemcpyDeviceToDevice, b->stream));
         StepArgs a = problem_args(b, p);
-        DevState ds;
-        if (e == cudaSuccess) e = cudaMemcpy(&ds, b->d_states + p, sizeof(ds), cudaMemcpyDeviceToHost);
-        a.t = ds.t;
+        a.ds = b->d_states + p;
+        a.dt_from_dev = 1;   // the time of its ghost data
         a.M = b->M_pending;
         a.pp_eps = b->pp_pending;
-        if (e == cudaSuccess)
-            e = crk::launch_limit2d(crk::PHYS_EULER, b->precision, b->k, b->basis, a, tmp, b->d_flags, b->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-        if (e == cudaSuccess) {
-            if (b->precision == CRKDG_F64) {
-                e = cudaMemcpy(h, tmp, n * 8, cudaMemcpyDeviceToHost);
-            } else {
-                std::vector<float> f(n);
-                e = cudaMemcpy(f.data(), tmp, n * 4, cudaMemcpyDeviceToHost);
-                for (size_t i = 0; i < n; ++i) h[i] = f[i];
-            }
-        }
-        cudaFree(tmp);
-        if (e != cudaSuccess) return bfail(CRKDG_ECUDA, std::string("get_state: ") + cudaGetErrorString(e));
-        return CRKDG_OK;
+        BCK(crk::launch_limit2d(crk::PHYS_EULER, b->precision, b->k, b->basis, a, tmp, b->d_flags, b->stream));
+        src = tmp;
     }
-    if (b->precision == CRKDG_F64) {
-        BCK(cudaMemcpy(h, base, n * 8, cudaMemcpyDeviceToHost));
-    } else {
-        std::vector<float> f(n);
-        BCK(cudaMemcpy(f.data(), base, n * 4, cudaMemcpyDeviceToHost));
-        for (size_t i = 0; i < n; ++i) h[i] = f[i];
+    if (f32) {   // widened on the GPU
+        BCK(crk::launch_f32_to_f64(static_cast<const float*>(src), b->d_stage, n, 0, b->stream));
+        src = b->d_stage;
     }
+    BCK(cudaMemcpyAsync(h, src, n * 8, cudaMemcpyDeviceToHost, b->stream));
+    BCK(cudaStreamSynchronize(b->stream));
     return CRKDG_OK;
 }
 
