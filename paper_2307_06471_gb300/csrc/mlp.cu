@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(REDUCE_RUNS * REDUCE_PARAMS)
 // samples' features as one run of memory and rounds them into its staging area
 // (VEC: pairs, where X allows 8-byte loads).  A block per 128 samples that
 // loaded the weights each time, lanes reading 160 bytes apart and the weights'
-// rows in one bank group took 0.202 ms for 524,288 samples; this takes 0.055 ms.
+// rows in one bank group took 0.202 ms for 524,288 samples; this takes 0.043 ms.
 constexpr int PREDICT_THREADS = 128;
 template <bool VEC>
 __global__ void __launch_bounds__(PREDICT_THREADS) mlp_predict_kernel(const float* __restrict__ prm,
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(PREDICT_THREADS) mlp_predict_kernel(const floa
             const int i = j * 32 + lane, r = i / PAIRS, k = 2 * (i % PAIRS);
             *reinterpret_cast<uint32_t*>(stage + r * crk::MLP_INP + k) = crk::pack_bf16(f[j].x, f[j].y);
         }
-        const float z = crk::mlp_warp_staged(w, stage);
+        const float z = crk::mlp_warp_staged2(w, stage);
         if (lane < ns) logits[s0 + lane] = z;
     }
 }

@@ -71,6 +71,88 @@ __device__ __forceinline__ void mlp_layer(const uint32_t (&a)[KS][4], const __nv
     }
 }
 
+// One hidden layer of both of the warp's 16-row tiles: a weight fragment is
+// loaded once for the two (twice the accumulator registers of mlp_layer)
+template <int KS, bool SWZ>
+__device__ __forceinline__ void mlp_layer2(const uint32_t (&a)[2][KS][4], const __nv_bfloat16* W, const float* bias,
+                                           int ldw, float (&acc)[2][8][4], int g, int tig) {
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+        const float b0 = bias[nt * 8 + 2 * tig], b1 = bias[nt * 8 + 2 * tig + 1];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+            acc[mt][nt][0] = acc[mt][nt][2] = b0;
+            acc[mt][nt][1] = acc[mt][nt][3] = b1;
+        }
+        const __nv_bfloat16* wr = W + (size_t)(nt * 8 + g) * ldw;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+            const int k0 = SWZ ? mlp_swz(g, ks * 16) : ks * 16, k1 = SWZ ? mlp_swz(g, ks * 16 + 8) : ks * 16 + 8;
+            const uint32_t bb0 = *reinterpret_cast<const uint32_t*>(wr + k0 + 2 * tig);
+            const uint32_t bb1 = *reinterpret_cast<const uint32_t*>(wr + k1 + 2 * tig);
+            mma_bf16(acc[0][nt], a[0][ks], bb0, bb1);
+            mma_bf16(acc[1][nt], a[1][ks], bb0, bb1);
+        }
+    }
+}
+
+// mlp_warp_staged for kernels with registers to spare: the same products in
+// the same order, both tiles at once.  The shared-memory reads of the weight
+// fragments bound the inference of mlp.cu: 0.055 ms for 524,288 samples tile
+// by tile, 0.043 so.
+__device__ __forceinline__ float mlp_warp_staged2(const MlpSmem& w, __nv_bfloat16* stage) {
+    const int lane = threadIdx.x & 31;
+    const int g = lane >> 2, tig = lane & 3;
+    float* lout = reinterpret_cast<float*>(stage + 32 * MLP_INP);
+    __syncwarp();
+    uint32_t a1[2][3][4], ah[2][4][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+        const __nv_bfloat16* r0 = stage + (mt * 16 + g) * MLP_INP;
+        const __nv_bfloat16* r1 = stage + (mt * 16 + g + 8) * MLP_INP;
+#pragma unroll
+        for (int ks = 0; ks < 3; ++ks) {
+            a1[mt][ks][0] = *reinterpret_cast<const uint32_t*>(r0 + ks * 16 + 2 * tig);
+            a1[mt][ks][1] = *reinterpret_cast<const uint32_t*>(r1 + ks * 16 + 2 * tig);
+            a1[mt][ks][2] = *reinterpret_cast<const uint32_t*>(r0 + ks * 16 + 8 + 2 * tig);
+            a1[mt][ks][3] = *reinterpret_cast<const uint32_t*>(r1 + ks * 16 + 8 + 2 * tig);
+        }
+    }
+    float acc[2][8][4];
+    auto next = [&]() {
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) c_to_a(acc[mt][2 * t], acc[mt][2 * t + 1], ah[mt][t]);
+    };
+    mlp_layer2<3, false>(a1, w.W1, w.b1, MLP_INP, acc, g, tig);
+    next();
+    mlp_layer2<4, true>(ah, w.W2, w.b2, MLP_H, acc, g, tig);
+    next();
+    mlp_layer2<4, true>(ah, w.W3, w.b3, MLP_H, acc, g, tig);
+    next();
+    // output layer: one 8-column tile, column 0 is the logit
+    const __nv_bfloat16* wr = w.W4 + (size_t)g * MLP_H;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+        float o[4] = {w.b4[2 * tig], w.b4[2 * tig + 1], w.b4[2 * tig], w.b4[2 * tig + 1]};
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+            const uint32_t bb0 = *reinterpret_cast<const uint32_t*>(wr + mlp_swz(g, ks * 16) + 2 * tig);
+            const uint32_t bb1 = *reinterpret_cast<const uint32_t*>(wr + mlp_swz(g, ks * 16 + 8) + 2 * tig);
+            mma_bf16(o, ah[mt][ks], bb0, bb1);
+        }
+        if (tig == 0) {
+            lout[mt * 16 + g] = o[0];
+            lout[mt * 16 + g + 8] = o[2];
+        }
+    }
+    __syncwarp();
+    const float z = lout[lane];
+    __syncwarp();
+    return z;
+}
+
 // Logits of the 32 cells whose features fill the warp's 32 x 48 BF16 staging
 // area (+ 32 floats after it); lane l returns cell l's.
 __device__ __forceinline__ float mlp_warp_staged(const MlpSmem& w, __nv_bfloat16* stage) {
