@@ -467,13 +467,21 @@ __device__ __forceinline__ LimMesh single_mesh(const StepArgs& a) {
     return g;
 }
 
+// Resident blocks per SM the pass is compiled for.  FP64: a cell's values alone
+// fill 56 of the 72 registers 7 blocks leave a thread: 0.103 ms per pass on the
+// 640x160 P^2 state, 0.094 at 4 blocks (128 registers).
+template <class T>
+constexpr int limit_minb() {
+    return sizeof(T) == 4 ? CRK_LIMIT_MINB : 4;
+}
+
 // The limiter pass: 128 threads per block along x, one block row per mesh
 // row.  Counts troubled cells (one atomic per warp that has any).  7 blocks
 // per SM (72 registers, a few bytes of spills): on the 1920x480 P^2 state
 // 0.0306 ms per pass against 0.0311 at 6 blocks (80 registers, none); 8
 // blocks spill more and measured slower, 5 slower still.
 template <class T, int K, int B, int PHYS>
-__global__ void __launch_bounds__(128, CRK_LIMIT_MINB) limit2d_kernel(const StepArgs a, T* __restrict__ u,
+__global__ void __launch_bounds__(128, limit_minb<T>()) limit2d_kernel(const StepArgs a, T* __restrict__ u,
                                                                       unsigned long long* flag_count) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const bool fl = limit2d_cell<T, K, B, PHYS, 0>(a, single_mesh<T>(a), u, x, blockIdx.y, nullptr, nullptr);
@@ -544,7 +552,7 @@ __global__ void __launch_bounds__(MLPTC_CELLS) limit2d_mlp_tc_kernel(const StepA
 // current buffer limited in place; problems that reached t_end (dt 0) are
 // left as they are.  Troubled cells count into the problem's run state.
 template <class T, int K, int B>
-__global__ void __launch_bounds__(128, CRK_LIMIT_MINB)
+__global__ void __launch_bounds__(128, limit_minb<T>())
     batch_limit2d_kernel(const StepArgs a, const BatchProblem* __restrict__ probs, const int4* __restrict__ rows,
                          DevState* states, const int* curs, T* bufA, T* bufB) {
     const int4 rt = rows[blockIdx.x];
