@@ -135,10 +135,10 @@ void strips_segs(const crkdg_ctx* c, int seg_rows, int* ns, int* nseg) {
     *nseg = (c->mesh.ny + seg_rows - 1) / seg_rows;
 }
 
-// bytes of one segment's seam scratch (2D quadrature step)
-size_t seam_seg_bytes(const crkdg_ctx* c) {
-    return crk::seam_values(c->tab.s, c->k + 1, c->nv, c->nm, c->precision == CRKDG_F32D,
-                            c->limit_mode == CRKDG_LIMIT_FUSED, c->mesh.nx) * c->esize;
+// bytes of one segment's seam scratch (2D quadrature step); `fused`: the pending
+// limit runs on load and its limited rows are kept too
+size_t seam_seg_bytes(const crkdg_ctx* c, bool fused) {
+    return crk::seam_values(c->tab.s, c->k + 1, c->nv, c->nm, c->precision == CRKDG_F32D, fused, c->mesh.nx) * c->esize;
 }
 // whether the quadrature step leaves the faces between its segments to the
 // seam launches (the compensated state without
@@ -148,10 +148,13 @@ bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load) {
 }
 
 // launch geometry of the quadrature step (its scratch bounds the segments)
-void step_segs(const crkdg_ctx* c, int* ns, int* nseg) {
+void step_segs(const crkdg_ctx* c, bool fused, int* ns, int* nseg) {
     strips_segs(c, c->seg_rows, ns, nseg);
     if (step_seams(c, *nseg, false))
-        *nseg = crk::seam_segments(*nseg, seam_seg_bytes(c), c->elems * c->esize * c->planes);
+        *nseg = crk::seam_segments(*nseg, seam_seg_bytes(c, fused), c->elems * c->esize * c->planes);
+}
+void step_segs(const crkdg_ctx* c, int* ns, int* nseg) {
+    step_segs(c, c->limit_mode == CRKDG_LIMIT_FUSED, ns, nseg);
 }
 
 int ensure_partials(crkdg_ctx* c, size_t n) {
@@ -163,13 +166,19 @@ int ensure_partials(crkdg_ctx* c, size_t n) {
     return CRKDG_OK;
 }
 
-// the quadrature step's scratch: reduction slots and seams
+// the quadrature step's scratch, reduction slots and seams: for either limit
+// mode, so that changing the mode moves no buffer a caller's graph may hold
 int ensure_step_scratch(crkdg_ctx* c) {
-    int ns, nseg;
-    step_segs(c, &ns, &nseg);
-    int r = ensure_partials(c, ((size_t)ns * nseg + crk::seam_blocks(c->nv, c->mesh.nx, c->mesh.ny, nseg, 2 * std::max(1, crk::sm_count()))) * (c->nv + 2));
+    size_t slots = 0, need = 0;
+    for (const bool fused : {false, true}) {
+        int ns, nseg;
+        step_segs(c, fused, &ns, &nseg);
+        const int tail = crk::seam_blocks(c->nv, c->mesh.nx, c->mesh.ny, nseg, 2 * std::max(1, crk::sm_count()));
+        slots = std::max(slots, (size_t)ns * nseg + tail);
+        if (step_seams(c, nseg, false)) need = std::max(need, seam_seg_bytes(c, fused) * nseg);
+    }
+    int r = ensure_partials(c, slots * (c->nv + 2));
     if (r) return r;
-    const size_t need = step_seams(c, nseg, false) ? seam_seg_bytes(c) * nseg : 0;
     if (need <= c->seam_cap) return CRKDG_OK;
     if (c->d_seam) cudaFree(c->d_seam);
     c->d_seam = nullptr;
@@ -295,6 +304,25 @@ int linear_shape(crkdg_ctx* c) {
     return CRKDG_OK;
 }
 
+// the modal step's scratch: reduction slots and boundary data
+int ensure_linear_scratch(crkdg_ctx* c) {
+    int r = linear_shape(c);
+    if (r) return r;
+    int ns, nseg;
+    strips_segs(c, c->lin_seg_rows, &ns, &nseg);
+    return ensure_partials(c, (size_t)ns * nseg * 8);
+}
+
+// the scratch of this context's 2D steps, made where their shape is set: a step
+// allocates nothing (it may be captured); the quadrature step's too where a
+// pending limit fused into the load can take a linear flux there
+int ensure_scratch(crkdg_ctx* c) {
+    if (c->dim != 2) return CRKDG_OK;
+    int r = use_linear(c) ? ensure_linear_scratch(c) : CRKDG_OK;
+    if (r || (use_linear(c) && c->limit_mode != CRKDG_LIMIT_FUSED)) return r;
+    return ensure_step_scratch(c);
+}
+
 // constants of the modal step: gamma_l = b^T A^l 1 of the tableau (FP64, host)
 // and the inflow faces
 void set_linear(const crkdg_ctx* c, StepArgs& a) {
@@ -363,16 +391,17 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
     a.M = M;
     a.pp_eps = limit ? c->pp_pending : 0.0;
     if (c->dim == 2) {
+        const bool fused = limit && c->limit_mode == CRKDG_LIMIT_FUSED;
         int ns, nseg;
         step_segs(c, &ns, &nseg);
         a.seg_len = c->seg_rows;
         a.n_strips = ns;
         a.n_segs = nseg;
-        int r = ensure_step_scratch(c);
+        int r = use_linear(c) && !fused ? ensure_linear_scratch(c) : ensure_step_scratch(c);
         if (r) return r;
         a.partials = c->d_partials;
         a.seam = c->d_seam;
-        a.seams = step_seams(c, nseg, a.limit && c->limit_mode == CRKDG_LIMIT_FUSED);
+        a.seams = step_seams(c, nseg, fused);
         if (c->mlp && limit && M >= 0.0 && c->limit_mode == CRKDG_LIMIT_FUSED) {
             a.mlp = c->mlp;
             a.mlp_zlo = c->mlp_zlo;
@@ -387,16 +416,8 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
                 a.limit = 0;
             }
             if (!a.limit && use_linear(c)) {
-                int r = linear_shape(c);
-                if (r) return r;
-                int lns, lnseg;
-                strips_segs(c, c->lin_seg_rows, &lns, &lnseg);
                 a.seg_len = c->lin_seg_rows;
-                a.n_strips = lns;
-                a.n_segs = lnseg;
-                r = ensure_partials(c, (size_t)lns * lnseg * 8);
-                if (r) return r;
-                a.partials = c->d_partials;
+                strips_segs(c, c->lin_seg_rows, &a.n_strips, &a.n_segs);
                 a.lin_data = c->d_lin_data;
                 set_linear(c, a);
                 CK(crk::launch_step2d_linear(c->precision, c->k, c->basis, a, c->lin_wpb, c->stream));
@@ -536,13 +557,8 @@ int create_impl(const crkdg_mesh* mesh, int k, int basis, int flux, const crkdg_
     if (r) return bail(r);
     r = default_launch(c);
     if (r) return bail(r);
-    if (c->dim == 2 && !use_linear(c)) {   // a step allocates nothing
-        r = ensure_step_scratch(c);
-        if (r) return bail(r);
-    } else if (c->dim == 2) {
-        r = linear_shape(c);
-        if (r) return bail(r);
-    }
+    r = ensure_scratch(c);
+    if (r) return bail(r);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return bail(fail(CRKDG_ECUDA, "stream sync failed"));
     *out = c;
     return CRKDG_OK;
@@ -772,16 +788,8 @@ int crkdg_advance(crkdg_ctx* c, int n_steps, double cfl, double t_end, int captu
     const int lim_rest = (c->limiter_on || c->pp_eps > 0.0) ? 1 : 0;
     const double M_first = c->M_pending, M_rest = c->M;
     const double pp_first = c->pp_pending, pp_rest = c->pp_eps;
-    r = ensure_step_scratch(c);
+    r = ensure_scratch(c);   // nothing may allocate while a graph is captured
     if (r) return r;
-    if (use_linear(c)) {   // slots of the modal step too: nothing may allocate while a graph is captured
-        r = linear_shape(c);
-        if (r) return r;
-        int ns, nseg;
-        strips_segs(c, c->lin_seg_rows, &ns, &nseg);
-        r = ensure_partials(c, (size_t)ns * nseg * 8);
-        if (r) return r;
-    }
     auto enqueue_all = [&]() -> int {
         for (int i = 0; i < n_steps; ++i) {
             const int lim = i == 0 ? lim_first : lim_rest;
@@ -1109,7 +1117,7 @@ int crkdg_set_launch(crkdg_ctx* c, int seg_rows, int wpb) {
     if (seg_rows > 0) c->seg_rows = std::min(seg_rows, c->mesh.ny);
     for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
     c->graphs.clear();
-    return CRKDG_OK;
+    return ensure_scratch(c);
 }
 
 int crkdg_apply_limit(crkdg_ctx* c) {
@@ -1127,7 +1135,7 @@ int crkdg_set_limit_mode(crkdg_ctx* c, int mode) {
     c->limit_mode = mode;
     for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
     c->graphs.clear();
-    return CRKDG_OK;
+    return ensure_scratch(c);
 }
 
 int crkdg_set_operator_form(crkdg_ctx* c, int form) {
@@ -1136,7 +1144,7 @@ int crkdg_set_operator_form(crkdg_ctx* c, int form) {
     c->op_form = form;
     for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
     c->graphs.clear();
-    return CRKDG_OK;
+    return ensure_scratch(c);
 }
 
 int crkdg_get_operator_form(const crkdg_ctx* c, int* form) {

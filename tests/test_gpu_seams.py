@@ -97,3 +97,46 @@ def test_batch_segments(prec, basis, tab):
     for o in outs[1:]:
         for x, y in zip(o, outs[0]):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("case", ["mode", "linear"])
+def test_first_step_can_be_captured(case):
+    """A step allocates nothing: the first one on a context, and the first
+    after a change of the limit mode, are captured on the caller's stream; a
+    graph captured in the other mode stays valid.  Bitwise equal to steps that
+    are not captured."""
+    import torch
+    from paper_2307_06471_gb300 import binding as B
+    from paper_2307_06471_gb300 import tableaux as T
+    phys = "euler" if case == "mode" else "advection"
+    nx, ny = 333, 200
+    mesh = B.make_mesh(2, nx, ny, (0.0, 1.0, 0.0, 0.6), [B.BC_PERIODIC] * 4)
+    u = to_planes(inp.random_modal_state(ny, nx, 2, "P", phys, seed=9))
+    dt = 0.02 / nx
+    torch.zeros(1, device="cuda")
+    stream = torch.cuda.Stream()
+
+    def solver():
+        s = B.Solver(mesh, 2, B.BASIS_P, T.SSPRK3, B.EULER if case == "mode" else B.ADVECTION, B.F64, stream=stream.cuda_stream)
+        s.set_state(u, 0.0)
+        return s
+    plain, captured = solver(), solver()
+    graphs = []
+    for mode in ((B.LIMIT_PASS, B.LIMIT_FUSED) if case == "mode" else (B.LIMIT_PASS, B.LIMIT_PASS)):
+        for s in (plain, captured):
+            if case == "mode":
+                s.set_limit_mode(mode)
+                s.limit(50.0)
+        plain.step(dt)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            captured.step(dt)
+        graphs.append(g)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for g in graphs:
+            g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(captured.get_state(), plain.get_state())
+    captured.close()
+    plain.close()
