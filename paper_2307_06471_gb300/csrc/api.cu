@@ -144,7 +144,8 @@ size_t seam_seg_bytes(const crkdg_ctx* c, bool fused) {
 // seam launches (the compensated state without
 // deviation fluxes recomputes halo rows)
 bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load) {
-    return c->precision != CRKDG_F32C && crk::use_seams(c->esize, c->tab.s, c->nm, lim_on_load, c->mesh.ny, nseg);
+    return c->precision != CRKDG_F32C && crk::use_seams(c->esize, c->tab.s, c->nm, c->precision == CRKDG_F32D, lim_on_load,
+                                                             c->mesh.ny, nseg);
 }
 
 // launch geometry of the quadrature step (its scratch bounds the segments)

@@ -139,7 +139,7 @@ int build_tasks(crkdg_batch* b) {
     b->tasks.clear();
     b->flux.clear();
     b->seams.clear();
-    b->use_seams = crk::use_seams(b->esize, b->tab.s, b->nm, false, b->seg_rows, 1);
+    b->use_seams = crk::use_seams(b->esize, b->tab.s, b->nm, false, false, b->seg_rows, 1);
     int warp0 = 0;
     long long slots = 0, seam = 0;
     const size_t room = (size_t)256 << 20;
