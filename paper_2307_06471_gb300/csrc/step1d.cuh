@@ -245,6 +245,10 @@ __global__ void __launch_bounds__(256) step1d_kernel(const StepArgs a, int n_ste
     }
     const T rx = sizeof(T) == 4 ? T(a.rxf) : T(a.rx);
     const T* src = static_cast<const T*>(a.uin);
+    const auto cluster = cooperative_groups::this_cluster();
+    // a block's shared memory may be written once the block has started: every
+    // block says so here, and the first push waits for all of them
+    if (n_steps > 1) cluster.barrier_arrive();
     T un[NV][NM], out[NV][NM];
 #pragma unroll
     for (int v = 0; v < NV; ++v)
@@ -260,7 +264,7 @@ __global__ void __launch_bounds__(256) step1d_kernel(const StepArgs a, int n_ste
             else step1d_cell<T, K, PHYS, NV, NM>(a, ln, ph, t0, a.dt, rx, slot, un, out);
         }
         if (step + 1 == n_steps) break;
-        const auto cluster = cooperative_groups::this_cluster();
+        if (step == 0) cluster.barrier_wait();
         auto push = [&](int warp, int side) {   // to a warp's halo lane
             T* h = cluster.map_shared_rank(&halo[step & 1][warp % wpb][side][0], warp / wpb);
 #pragma unroll
