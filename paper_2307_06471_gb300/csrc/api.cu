@@ -158,29 +158,114 @@ void step_segs(const crkdg_ctx* c, int* ns, int* nseg) {
     step_segs(c, c->limit_mode == CRKDG_LIMIT_FUSED, ns, nseg);
 }
 
+// The graphs of earlier runs are recorded again: a launch shape changed, or
+// scratch that their launches write has moved
+void drop_graphs(crkdg_ctx* c) {
+    for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
+    c->graphs.clear();
+}
+
 int ensure_partials(crkdg_ctx* c, size_t n) {
     if (n <= c->partials_cap) return CRKDG_OK;
+    drop_graphs(c);
     if (c->d_partials) cudaFree(c->d_partials);
     c->d_partials = nullptr;
-    CK(cudaMalloc(&c->d_partials, n * sizeof(double)));
+    c->partials_cap = 0;
+    if (cudaMalloc(&c->d_partials, n * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        c->d_partials = nullptr;
+        return fail(CRKDG_ENOMEM, "cudaMalloc of the reduction slots failed");
+    }
     c->partials_cap = n;
     return CRKDG_OK;
+}
+
+// the modal step can take the context's steps: linear flux, 2D, FP32/FP64,
+// every non-periodic side affine (outflow, wall, constant state) or sine data
+bool linear_sides(const crkdg_ctx* c) {
+    if (c->kphys != crk::PHYS_ADV || c->dim != 2 || compensated(c->precision)) return false;
+    crk::BCSide bc[4];
+    for (int s = 0; s < 4; ++s) {
+        bc[s].type = c->mesh.bc[s];
+        bc[s].fn = c->mesh.bc_fn[s];
+        for (int j = 0; j < 16; ++j) bc[s].p[j] = c->mesh.bc_params[s][j];
+    }
+    crk::set_bc_affine(bc, 1);
+    for (int s = 0; s < 4; ++s)
+        if (bc[s].type != crk::BC_PERIODIC && !bc[s].affine &&
+            !(bc[s].type == crk::BC_DIRICHLET && (bc[s].fn == crk::FN_SINE || bc[s].fn == crk::FN_SINE_PROD)))
+            return false;
+    return true;
+}
+
+// ... and does: it is not switched off
+bool use_linear(const crkdg_ctx* c) { return c->op_form == CRKDG_FORM_AUTO && linear_sides(c); }
+
+// one wave of the modal step: as many warps as its registers and shared
+// memory let the device's SMs hold, segments of >= 1 row
+int linear_shape(crkdg_ctx* c) {
+    if (c->lin_seg_rows > 0) return CRKDG_OK;
+    // the boundary faces' data
+    const size_t data = (size_t)2 * (c->mesh.nx + c->mesh.ny) * (c->k + 1) * c->esize;
+    if (!c->d_lin_data && cudaMalloc(&c->d_lin_data, data) != cudaSuccess) {
+        cudaGetLastError();
+        c->d_lin_data = nullptr;
+        return fail(CRKDG_ENOMEM, "cudaMalloc of the boundary data failed");
+    }
+    crk::KernelInfo ki;
+    CK(crk::info_step2d_linear(c->precision, c->k, c->basis, &ki));
+    const int wpb = std::max(1, std::min(4, ki.max_threads / 32));
+    const int regs_warp = ((ki.regs + 7) / 8) * 8 * 32;
+    const int by_regs = 65536 / regs_warp;
+    const int by_smem = (228 * 1024) / std::max(1, ki.smem_per_thread * 32);
+    int resident = std::min(64, std::min(by_regs, by_smem));
+    resident = std::max(wpb, resident / wpb * wpb);
+    const int ns = (c->mesh.nx + 29) / 30;
+    const long nseg = std::max(1L, (long)std::max(1, crk::sm_count()) * resident / ns);
+    const int L = (int)std::max(1L, ((long)c->mesh.ny + nseg - 1) / nseg);
+    c->lin_seg_rows = std::min(L, c->mesh.ny);
+    c->lin_wpb = wpb;
+    // few warps: blocks small enough to reach every SM
+    const long warps = (long)ns * ((c->mesh.ny + c->lin_seg_rows - 1) / c->lin_seg_rows);
+    while (c->lin_wpb > 1 && warps < (long)c->lin_wpb * crk::sm_count()) c->lin_wpb /= 2;
+    return CRKDG_OK;
+}
+
+// Reduction slots for every launch of the context -- the reductions of the
+// averages, the step in either limit mode and operator form -- so that no call
+// between two others moves the buffer their launches, or a graph of them, hold
+int ensure_slots(crkdg_ctx* c) {
+    size_t n = (size_t)crk::reduce_blocks(c->ncell, crk::sm_count()) * crk::REDUCE_SLOT;
+    if (c->dim == 2) {
+        int ns, nseg;
+        for (const bool fused : {false, true}) {
+            step_segs(c, fused, &ns, &nseg);
+            const int tail = crk::seam_blocks(c->nv, c->mesh.nx, c->mesh.ny, nseg, 2 * std::max(1, crk::sm_count()));
+            n = std::max(n, ((size_t)ns * nseg + tail) * (c->nv + 2));
+        }
+        if (linear_sides(c)) {
+            int r = linear_shape(c);
+            if (r) return r;
+            strips_segs(c, c->lin_seg_rows, &ns, &nseg);
+            n = std::max(n, (size_t)ns * nseg * (c->nv + 2));
+        }
+    }
+    return ensure_partials(c, n);
 }
 
 // the quadrature step's scratch, reduction slots and seams: for either limit
 // mode, so that changing the mode moves no buffer a caller's graph may hold
 int ensure_step_scratch(crkdg_ctx* c) {
-    size_t slots = 0, need = 0;
+    int r = ensure_slots(c);
+    if (r) return r;
+    size_t need = 0;
     for (const bool fused : {false, true}) {
         int ns, nseg;
         step_segs(c, fused, &ns, &nseg);
-        const int tail = crk::seam_blocks(c->nv, c->mesh.nx, c->mesh.ny, nseg, 2 * std::max(1, crk::sm_count()));
-        slots = std::max(slots, (size_t)ns * nseg + tail);
         if (step_seams(c, nseg, false)) need = std::max(need, seam_seg_bytes(c, fused) * nseg);
     }
-    int r = ensure_partials(c, slots * (c->nv + 2));
-    if (r) return r;
     if (need <= c->seam_cap) return CRKDG_OK;
+    drop_graphs(c);
     if (c->d_seam) cudaFree(c->d_seam);
     c->d_seam = nullptr;
     c->seam_cap = 0;
@@ -247,7 +332,7 @@ int default_launch(crkdg_ctx* c) {
 int enqueue_reduce(crkdg_ctx* c, crk::ReduceRun run) {
     run.set_estimate(c->gamma, dx_of(c), dy_of(c));
     const int blocks = crk::reduce_blocks(c->ncell, crk::sm_count());
-    int r = ensure_partials(c, (size_t)blocks * crk::REDUCE_SLOT);
+    int r = ensure_slots(c);
     if (r) return r;
     CK(crk::launch_reduce(c->dim, c->kphys, c->precision, c->u[c->cur], c->mesh.nx, c->dim == 1 ? 1 : c->mesh.ny, c->nm,
                           dx_of(c), dy_of(c), c->gamma, c->beta[0], c->beta[1], c->d_state, c->d_partials, blocks,
@@ -255,72 +340,12 @@ int enqueue_reduce(crkdg_ctx* c, crk::ReduceRun run) {
     return CRKDG_OK;
 }
 
-// the modal step applies: linear flux, 2D, FP32/FP64, every non-periodic side
-// affine (outflow, wall, constant state) or sine data, not switched off
-bool use_linear(const crkdg_ctx* c) {
-    if (c->op_form != CRKDG_FORM_AUTO || c->kphys != crk::PHYS_ADV || c->dim != 2 ||
-        compensated(c->precision))
-        return false;
-    crk::BCSide bc[4];
-    for (int s = 0; s < 4; ++s) {
-        bc[s].type = c->mesh.bc[s];
-        bc[s].fn = c->mesh.bc_fn[s];
-        for (int j = 0; j < 16; ++j) bc[s].p[j] = c->mesh.bc_params[s][j];
-    }
-    crk::set_bc_affine(bc, 1);
-    for (int s = 0; s < 4; ++s)
-        if (bc[s].type != crk::BC_PERIODIC && !bc[s].affine &&
-            !(bc[s].type == crk::BC_DIRICHLET && (bc[s].fn == crk::FN_SINE || bc[s].fn == crk::FN_SINE_PROD)))
-            return false;
-    return true;
-}
-
-// one wave of the modal step: as many warps as its registers and shared
-// memory let the device's SMs hold, segments of >= 1 row
-int linear_shape(crkdg_ctx* c) {
-    if (c->lin_seg_rows > 0) return CRKDG_OK;
-    // the boundary faces' data
-    const size_t data = (size_t)2 * (c->mesh.nx + c->mesh.ny) * (c->k + 1) * c->esize;
-    if (!c->d_lin_data && cudaMalloc(&c->d_lin_data, data) != cudaSuccess) {
-        cudaGetLastError();
-        c->d_lin_data = nullptr;
-        return fail(CRKDG_ENOMEM, "cudaMalloc of the boundary data failed");
-    }
-    crk::KernelInfo ki;
-    CK(crk::info_step2d_linear(c->precision, c->k, c->basis, &ki));
-    const int wpb = std::max(1, std::min(4, ki.max_threads / 32));
-    const int regs_warp = ((ki.regs + 7) / 8) * 8 * 32;
-    const int by_regs = 65536 / regs_warp;
-    const int by_smem = (228 * 1024) / std::max(1, ki.smem_per_thread * 32);
-    int resident = std::min(64, std::min(by_regs, by_smem));
-    resident = std::max(wpb, resident / wpb * wpb);
-    const int ns = (c->mesh.nx + 29) / 30;
-    const long nseg = std::max(1L, (long)std::max(1, crk::sm_count()) * resident / ns);
-    const int L = (int)std::max(1L, ((long)c->mesh.ny + nseg - 1) / nseg);
-    c->lin_seg_rows = std::min(L, c->mesh.ny);
-    c->lin_wpb = wpb;
-    // few warps: blocks small enough to reach every SM
-    const long warps = (long)ns * ((c->mesh.ny + c->lin_seg_rows - 1) / c->lin_seg_rows);
-    while (c->lin_wpb > 1 && warps < (long)c->lin_wpb * crk::sm_count()) c->lin_wpb /= 2;
-    return CRKDG_OK;
-}
-
-// the modal step's scratch: reduction slots and boundary data
-int ensure_linear_scratch(crkdg_ctx* c) {
-    int r = linear_shape(c);
-    if (r) return r;
-    int ns, nseg;
-    strips_segs(c, c->lin_seg_rows, &ns, &nseg);
-    return ensure_partials(c, (size_t)ns * nseg * 8);
-}
-
-// the scratch of this context's 2D steps, made where their shape is set: a step
-// allocates nothing (it may be captured); the quadrature step's too where a
-// pending limit fused into the load can take a linear flux there
+// the scratch of this context's steps, made where their shape is set: a step
+// allocates nothing (it may be captured).  The modal step takes no seams; a
+// linear flux has theirs where a pending limit fused into the load sends it to
+// the quadrature step (and from its first crkdg_rkdg_step on).
 int ensure_scratch(crkdg_ctx* c) {
-    if (c->dim != 2) return CRKDG_OK;
-    int r = use_linear(c) ? ensure_linear_scratch(c) : CRKDG_OK;
-    if (r || (use_linear(c) && c->limit_mode != CRKDG_LIMIT_FUSED)) return r;
+    if (c->dim != 2 || (use_linear(c) && c->limit_mode != CRKDG_LIMIT_FUSED)) return ensure_slots(c);
     return ensure_step_scratch(c);
 }
 
@@ -398,7 +423,7 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
         a.seg_len = c->seg_rows;
         a.n_strips = ns;
         a.n_segs = nseg;
-        int r = use_linear(c) && !fused ? ensure_linear_scratch(c) : ensure_step_scratch(c);
+        int r = use_linear(c) && !fused ? ensure_slots(c) : ensure_step_scratch(c);
         if (r) return r;
         a.partials = c->d_partials;
         a.seam = c->d_seam;
@@ -1024,8 +1049,7 @@ int crkdg_set_indicator_engine(crkdg_ctx* c, int engine) {
     if (engine != CRKDG_MLP_TCGEN05 && engine != CRKDG_MLP_MMA_SYNC)
         return fail(CRKDG_EINVAL, "unknown indicator engine");
     c->mlp_engine = engine;
-    for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
-    c->graphs.clear();
+    drop_graphs(c);
     return CRKDG_OK;
 }
 
@@ -1116,8 +1140,7 @@ int crkdg_set_launch(crkdg_ctx* c, int seg_rows, int wpb) {
         c->wpb = wpb;
     }
     if (seg_rows > 0) c->seg_rows = std::min(seg_rows, c->mesh.ny);
-    for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
-    c->graphs.clear();
+    drop_graphs(c);
     return ensure_scratch(c);
 }
 
@@ -1134,8 +1157,7 @@ int crkdg_set_limit_mode(crkdg_ctx* c, int mode) {
     if (check_ctx(c)) return CRKDG_EINVAL;
     if (mode != CRKDG_LIMIT_FUSED && mode != CRKDG_LIMIT_PASS) return fail(CRKDG_EINVAL, "unknown limit mode");
     c->limit_mode = mode;
-    for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
-    c->graphs.clear();
+    drop_graphs(c);
     return ensure_scratch(c);
 }
 
@@ -1143,8 +1165,7 @@ int crkdg_set_operator_form(crkdg_ctx* c, int form) {
     if (check_ctx(c)) return CRKDG_EINVAL;
     if (form != CRKDG_FORM_QUADRATURE && form != CRKDG_FORM_AUTO) return fail(CRKDG_EINVAL, "unknown operator form");
     c->op_form = form;
-    for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
-    c->graphs.clear();
+    drop_graphs(c);
     return ensure_scratch(c);
 }
 
@@ -1265,8 +1286,7 @@ int crkdg_autotune(crkdg_ctx* c, double* best_us) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     CK(cudaMemcpy(c->d_state, &saved, sizeof(DevState), cudaMemcpyHostToDevice));
-    for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
-    c->graphs.clear();
+    drop_graphs(c);
     if (best_us) *best_us = best;
     return CRKDG_OK;
 }
