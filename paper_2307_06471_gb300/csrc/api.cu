@@ -64,6 +64,8 @@ struct crkdg_ctx {
     size_t partials_cap;
     void* d_seam = nullptr;       // seam scratch of the 2D step
     size_t seam_cap = 0;          // its bytes
+    size_t seam_room = 0;         // what its segments may ask for (seam_room; less on a full device)
+    bool seams_off = false;       // FP32 on a full device: halo rows are recomputed instead
     unsigned long long* d_flags;
     cudaStream_t stream;
     double t;
@@ -144,7 +146,7 @@ size_t seam_seg_bytes(const crkdg_ctx* c, bool fused) {
 // seam launches (the compensated state without
 // deviation fluxes recomputes halo rows)
 bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load) {
-    return c->precision != CRKDG_F32C && crk::use_seams(c->esize, c->tab.s, c->nm, c->precision == CRKDG_F32D, lim_on_load,
+    return c->precision != CRKDG_F32C && !c->seams_off && crk::use_seams(c->esize, c->tab.s, c->nm, c->precision == CRKDG_F32D, lim_on_load,
                                                              c->mesh.ny, nseg);
 }
 
@@ -152,7 +154,7 @@ bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load) {
 void step_segs(const crkdg_ctx* c, bool fused, int* ns, int* nseg) {
     strips_segs(c, c->seg_rows, ns, nseg);
     if (step_seams(c, *nseg, false))
-        *nseg = crk::seam_segments(*nseg, seam_seg_bytes(c, fused), c->elems * c->esize * c->planes);
+        *nseg = crk::seam_segments(*nseg, seam_seg_bytes(c, fused), c->seam_room);
 }
 void step_segs(const crkdg_ctx* c, int* ns, int* nseg) {
     step_segs(c, c->limit_mode == CRKDG_LIMIT_FUSED, ns, nseg);
@@ -253,29 +255,53 @@ int ensure_slots(crkdg_ctx* c) {
     return ensure_partials(c, n);
 }
 
-// the quadrature step's scratch, reduction slots and seams: for either limit
-// mode, so that changing the mode moves no buffer a caller's graph may hold
-int ensure_step_scratch(crkdg_ctx* c) {
-    int r = ensure_slots(c);
-    if (r) return r;
+// the seam scratch the launch shape asks for, for either limit mode
+size_t seam_need(const crkdg_ctx* c) {
     size_t need = 0;
     for (const bool fused : {false, true}) {
         int ns, nseg;
         step_segs(c, fused, &ns, &nseg);
         if (step_seams(c, nseg, false)) need = std::max(need, seam_seg_bytes(c, fused) * nseg);
     }
-    if (need <= c->seam_cap) return CRKDG_OK;
+    return need;
+}
+void free_seam(crkdg_ctx* c) {
     drop_graphs(c);
     if (c->d_seam) cudaFree(c->d_seam);
     c->d_seam = nullptr;
     c->seam_cap = 0;
-    if (cudaMalloc(&c->d_seam, need) != cudaSuccess) {
+}
+// a new launch shape may ask for the whole room again
+void reset_seam_room(crkdg_ctx* c) {
+    c->seam_room = crk::seam_room(c->elems * c->esize * c->planes);
+    c->seams_off = false;
+}
+
+// the quadrature step's scratch, reduction slots and seams: for either limit
+// mode, so that changing the mode moves no buffer a caller's graph may hold.
+// Where the device has no room for it, fewer segments (FP64) or halo rows
+// (FP32): the segments do not change a result.
+int ensure_step_scratch(crkdg_ctx* c) {
+    for (;;) {
+        int r = ensure_slots(c);
+        if (r) return r;
+        const size_t need = seam_need(c);
+        if (need <= c->seam_cap) return CRKDG_OK;
+        free_seam(c);
+        if (cudaMalloc(&c->d_seam, need) == cudaSuccess) {
+            c->seam_cap = need;
+            return CRKDG_OK;
+        }
         cudaGetLastError();
         c->d_seam = nullptr;
-        return fail(CRKDG_ENOMEM, "cudaMalloc of the step's seam scratch failed");
+        if (c->esize == 4) {
+            c->seams_off = true;
+        } else if (need <= seam_seg_bytes(c, true)) {   // one segment
+            return fail(CRKDG_ENOMEM, "cudaMalloc of the step's seam scratch failed");
+        } else {
+            c->seam_room = need / 2;
+        }
     }
-    c->seam_cap = need;
-    return CRKDG_OK;
 }
 
 int max_wpb(crkdg_ctx* c) {
@@ -551,6 +577,7 @@ int create_impl(const crkdg_mesh* mesh, int k, int basis, int flux, const crkdg_
     c->M = -1.0;
     c->seg_rows = 8;
     c->wpb = 4;
+    reset_seam_room(c);
     auto bail = [&](int code) {
         crkdg_destroy(c);
         return code;
@@ -1141,6 +1168,7 @@ int crkdg_set_launch(crkdg_ctx* c, int seg_rows, int wpb) {
     }
     if (seg_rows > 0) c->seg_rows = std::min(seg_rows, c->mesh.ny);
     drop_graphs(c);
+    reset_seam_room(c);
     return ensure_scratch(c);
 }
 
@@ -1246,6 +1274,7 @@ int crkdg_autotune(crkdg_ctx* c, double* best_us) {
     double best = 1e30;
     int bl = c->seg_rows, bw = c->wpb;
     const int cur0 = c->cur;
+    const size_t seam_cap0 = c->seam_cap;
     double dt = 0.0;
     {
         int r = enqueue_reduce(c, {0, 0, 0.0, 0.0});
@@ -1259,6 +1288,7 @@ int crkdg_autotune(crkdg_ctx* c, double* best_us) {
             const int w = cw.second;
             c->seg_rows = cw.first;
             c->wpb = w;
+            reset_seam_room(c);
             float t[6];
             for (int it = 0; it < 6; ++it) {
                 c->cur = cur0;
@@ -1288,7 +1318,10 @@ int crkdg_autotune(crkdg_ctx* c, double* best_us) {
     CK(cudaMemcpy(c->d_state, &saved, sizeof(DevState), cudaMemcpyHostToDevice));
     drop_graphs(c);
     if (best_us) *best_us = best;
-    return CRKDG_OK;
+    // the scratch of the kept shape, not of the largest one tried
+    reset_seam_room(c);
+    if (c->seam_cap > seam_cap0) free_seam(c);
+    return ensure_scratch(c);
 }
 
 int crkdg_save(crkdg_ctx* c, const char* path) {

@@ -142,7 +142,6 @@ int build_tasks(crkdg_batch* b) {
     b->use_seams = crk::use_seams(b->esize, b->tab.s, b->nm, false, false, b->seg_rows, 1);
     int warp0 = 0;
     long long slots = 0, seam = 0;
-    const size_t room = (size_t)256 << 20;
     for (int p = 0; p < b->n; ++p) {
         BatchProblem& pb = b->probs[p];
         const size_t values = (size_t)pb.nx * pb.ny * b->nv * b->nm;
@@ -151,8 +150,9 @@ int build_tasks(crkdg_batch* b) {
         pb.n_strips = (pb.nx + 29) / 30;
         pb.n_segs = (pb.ny + b->seg_rows - 1) / b->seg_rows;
         if (b->use_seams)
-            pb.n_segs = crk::seam_segments(pb.n_segs, seg * b->esize, values * b->esize,
-                                           (size_t)((double)room * values / b->elems));
+            pb.n_segs = crk::seam_segments(
+                pb.n_segs, seg * b->esize,
+                crk::seam_room(values * b->esize, (size_t)((double)crk::SEAM_ROOM * values / b->elems)));
         pb.n_seam_blocks = crk::seam_blocks(b->nv, pb.nx, pb.ny, pb.n_segs, 32);
         pb.warp0 = warp0;
         pb.slot0 = slots;

@@ -414,11 +414,16 @@ inline bool use_seams(size_t esize, int stages, int modes, bool dev, bool lim_on
     const int rows = stages * modes >= 27 ? (dev ? 64 : 6) : (stages * modes >= 18 ? 1 : 0);
     return !lim_on_load && ny <= (long long)rows * n_segs;
 }
-// Segments that keep the seam scratch within an eighth of a state copy (or
-// 256 MiB): a launch shape asks for memory in proportion to its segments
-inline int seam_segments(int n_segs, size_t seg_bytes, size_t state_bytes, size_t room = (size_t)256 << 20) {
-    const size_t cap = state_bytes / 8 > room ? state_bytes / 8 : room;
-    const size_t most = cap / (seg_bytes ? seg_bytes : 1);
+// What the seam scratch may take: an eighth of a state copy, or 256 MiB.  A launch
+// shape asks for memory in proportion to its segments, which seam_segments keeps
+// within a room (at least one); where the device has less to give, the caller
+// halves the room.
+constexpr size_t SEAM_ROOM = (size_t)256 << 20;
+inline size_t seam_room(size_t state_bytes, size_t least = SEAM_ROOM) {
+    return state_bytes / 8 > least ? state_bytes / 8 : least;
+}
+inline int seam_segments(int n_segs, size_t seg_bytes, size_t room) {
+    const size_t most = room / (seg_bytes ? seg_bytes : 1);
     return (size_t)n_segs <= most ? n_segs : (most ? (int)most : 1);
 }
 
