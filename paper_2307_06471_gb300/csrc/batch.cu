@@ -94,6 +94,7 @@ struct crkdg_batch {
     std::vector<int2> tasks;
     std::vector<int2> flux, seams;         // the seam launches' blocks: (problem, block)
     bool use_seams = false;                // (use_seams)
+    bool ready = false;                    // the tables below are those of the launch shape
     void* buf[2] = {nullptr, nullptr};
     BatchProblem* d_probs = nullptr;
     int2* d_tasks = nullptr;
@@ -134,12 +135,24 @@ StepArgs batch_args(const crkdg_batch* b) {
     return a;
 }
 
-// rebuild the task table for the current segment length
-int build_tasks(crkdg_batch* b) {
+void free_tables(crkdg_batch* b) {
+    b->ready = false;
+    for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);   // they hold the tables
+    b->graphs.clear();
+    for (void** p : {(void**)&b->d_rows, (void**)&b->d_tasks, (void**)&b->d_flux, (void**)&b->d_seams, (void**)&b->d_seam,
+                     (void**)&b->d_partials}) {
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+}
+
+// the tables of the current segment length with at most `room` bytes of seam
+// scratch (shared among the problems by their size); returns the scratch's values
+size_t plan_tables(crkdg_batch* b, bool seams, size_t room, long long* n_slots) {
     b->tasks.clear();
     b->flux.clear();
     b->seams.clear();
-    b->use_seams = crk::use_seams(b->esize, b->tab.s, b->nm, false, false, b->seg_rows, 1);
+    b->use_seams = seams;
     int warp0 = 0;
     long long slots = 0, seam = 0;
     for (int p = 0; p < b->n; ++p) {
@@ -149,17 +162,14 @@ int build_tasks(crkdg_batch* b) {
                                             b->limit_mode == CRKDG_LIMIT_FUSED, pb.nx);
         pb.n_strips = (pb.nx + 29) / 30;
         pb.n_segs = (pb.ny + b->seg_rows - 1) / b->seg_rows;
-        if (b->use_seams)
-            pb.n_segs = crk::seam_segments(
-                pb.n_segs, seg * b->esize,
-                crk::seam_room(values * b->esize, (size_t)((double)crk::SEAM_ROOM * values / b->elems)));
+        if (seams) pb.n_segs = crk::seam_segments(pb.n_segs, seg * b->esize, (size_t)((double)room * values / b->elems));
         pb.n_seam_blocks = crk::seam_blocks(b->nv, pb.nx, pb.ny, pb.n_segs, 32);
         pb.warp0 = warp0;
         pb.slot0 = slots;
         pb.seam0 = seam;
         const int w = pb.n_strips * pb.n_segs;
         for (int i = 0; i < w; ++i) b->tasks.push_back(make_int2(p, i));
-        if (b->use_seams) {
+        if (seams) {
             const int nf = crk::seam_flux_blocks(b->esize, b->k + 1, pb.nx, pb.n_segs);
             for (int i = 0; i < nf; ++i) b->flux.push_back(make_int2(p, i));
             for (int i = 0; i < pb.n_seam_blocks; ++i) b->seams.push_back(make_int2(p, i));
@@ -168,40 +178,67 @@ int build_tasks(crkdg_batch* b) {
         warp0 += w;
         slots += w + pb.n_seam_blocks;
     }
+    *n_slots = slots;
+    return (size_t)seam;
+}
+
+// a table's device copy
+template <class V>
+int upload(V*& d, const std::vector<V>& h) {
+    if (h.empty()) return CRKDG_OK;
+    if (cudaMalloc(&d, h.size() * sizeof(V)) != cudaSuccess) {
+        cudaGetLastError();
+        d = nullptr;
+        return bfail(CRKDG_ENOMEM, "cudaMalloc of the batch's tables failed");
+    }
+    BCK(cudaMemcpy(d, h.data(), h.size() * sizeof(V), cudaMemcpyHostToDevice));
+    return CRKDG_OK;
+}
+
+// Rebuild the task tables for the current segment length.  Where the device has
+// no room for the seam scratch: halo rows (FP32) or fewer segments (FP64); a
+// batch whose tables could not be made runs nothing until they are.
+int build_tables(crkdg_batch* b) {
+    free_tables(b);
+    bool seams = crk::use_seams(b->esize, b->tab.s, b->nm, false, false, b->seg_rows, 1);
+    size_t room = crk::seam_room(b->elems * b->esize);
+    long long slots = 0;
+    for (;;) {
+        const size_t seam = plan_tables(b, seams, room, &slots);
+        if (!seam || cudaMalloc(&b->d_seam, seam * b->esize) == cudaSuccess) break;
+        cudaGetLastError();
+        b->d_seam = nullptr;
+        bool least = true;   // a segment a problem
+        for (const auto& pb : b->probs) least = least && pb.n_segs == 1;
+        if (b->esize == 4) seams = false;
+        else if (least) return bfail(CRKDG_ENOMEM, "cudaMalloc of the batch's seam scratch failed");
+        else room = std::min(room, seam * b->esize) / 2;
+    }
     // the limiter pass's tiles: 128 cells of one row of one problem
     std::vector<int4> rows;
     for (int p = 0; p < b->n; ++p)
         for (int y = 0; y < b->probs[p].ny; ++y)
             for (int x = 0; x < b->probs[p].nx; x += 128) rows.push_back(make_int4(p, y, x, 0));
-    if (b->d_tasks) cudaFree(b->d_tasks);
-    if (b->d_seam) cudaFree(b->d_seam);
-    if (b->d_flux) cudaFree(b->d_flux);
-    if (b->d_seams) cudaFree(b->d_seams);
-    if (b->d_partials) cudaFree(b->d_partials);
-    if (b->d_rows) cudaFree(b->d_rows);
-    b->d_tasks = nullptr;
-    b->d_seam = nullptr;
-    b->d_flux = nullptr;
-    b->d_seams = nullptr;
-    b->d_partials = nullptr;
-    b->d_rows = nullptr;
     b->n_rows = (int)rows.size();
-    BCK(cudaMalloc(&b->d_rows, rows.size() * sizeof(int4)));
-    BCK(cudaMemcpy(b->d_rows, rows.data(), rows.size() * sizeof(int4), cudaMemcpyHostToDevice));
-    BCK(cudaMalloc(&b->d_tasks, b->tasks.size() * sizeof(int2)));
-    BCK(cudaMalloc(&b->d_partials, std::max((size_t)slots * (b->nv + 2), (size_t)b->n * START_BLOCKS) * sizeof(double)));
-    BCK(cudaMemcpy(b->d_tasks, b->tasks.data(), b->tasks.size() * sizeof(int2), cudaMemcpyHostToDevice));
-    if (b->use_seams) {
-        BCK(cudaMalloc(&b->d_flux, b->flux.size() * sizeof(int2)));
-        BCK(cudaMalloc(&b->d_seams, b->seams.size() * sizeof(int2)));
-        BCK(cudaMalloc(&b->d_seam, (size_t)seam * b->esize));
-        BCK(cudaMemcpy(b->d_flux, b->flux.data(), b->flux.size() * sizeof(int2), cudaMemcpyHostToDevice));
-        BCK(cudaMemcpy(b->d_seams, b->seams.data(), b->seams.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    int r = upload(b->d_rows, rows);
+    if (!r) r = upload(b->d_tasks, b->tasks);
+    if (!r) r = upload(b->d_flux, b->flux);
+    if (!r) r = upload(b->d_seams, b->seams);
+    if (r) return r;
+    const size_t part = std::max((size_t)slots * (b->nv + 2), (size_t)b->n * START_BLOCKS);
+    if (cudaMalloc(&b->d_partials, part * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        b->d_partials = nullptr;
+        return bfail(CRKDG_ENOMEM, "cudaMalloc of the batch's reduction slots failed");
     }
     BCK(cudaMemcpy(b->d_probs, b->probs.data(), b->n * sizeof(BatchProblem), cudaMemcpyHostToDevice));
-    for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
-    b->graphs.clear();
+    b->ready = true;
     return CRKDG_OK;
+}
+int build_tasks(crkdg_batch* b) {
+    const int r = build_tables(b);
+    if (r) free_tables(b);
+    return r;
 }
 
 // Default launch shape: the shortest segments whose tasks the SMs hold at once,
@@ -544,8 +581,10 @@ int crkdg_batch_positivity(crkdg_batch* b, double eps) {
 int crkdg_batch_run(crkdg_batch* b, double cfl, double t_end, int steps_per_graph, int max_graphs, int* n_done) {
     if (!b || !(cfl > 0.0) || steps_per_graph < 1 || max_graphs < 1) return bfail(CRKDG_EINVAL, "bad argument");
     if (!b->stream) return bfail(CRKDG_EINVAL, "batched runs need a non-default stream (graph capture)");
+    int r0 = b->ready ? CRKDG_OK : build_tasks(b);
+    if (r0) return r0;
     BCK(cudaMemsetAsync(b->d_done, 0, sizeof(unsigned), b->stream));
-    int r0 = start_run(b, cfl, t_end);
+    r0 = start_run(b, cfl, t_end);
     if (r0) return r0;
     unsigned done = 0;
     for (int g = 0; g < max_graphs; ++g) {
@@ -606,7 +645,7 @@ int crkdg_batch_sizes(const crkdg_batch* b, int* n_problems, long long* total_ce
 int crkdg_batch_set_limit_mode(crkdg_batch* b, int mode) {
     if (!b) return bfail(CRKDG_EINVAL, "null batch");
     if (mode != CRKDG_LIMIT_FUSED && mode != CRKDG_LIMIT_PASS) return bfail(CRKDG_EINVAL, "unknown limit mode");
-    if (mode == b->limit_mode) return CRKDG_OK;
+    if (mode == b->limit_mode && b->ready) return CRKDG_OK;
     b->limit_mode = mode;
     return build_tasks(b);   // the seam scratch holds more in the fused mode
 }
@@ -622,7 +661,7 @@ int crkdg_batch_set_launch(crkdg_batch* b, int seg_rows, int wpb) {
             return bfail(CRKDG_EINVAL, "warps per block exceeds the kernel's limits");
         b->wpb = wpb;
     }
-    if (seg_rows > 0 && seg_rows != b->seg_rows) {
+    if (seg_rows > 0 && (seg_rows != b->seg_rows || !b->ready)) {
         b->seg_rows = seg_rows;
         return build_tasks(b);
     }
