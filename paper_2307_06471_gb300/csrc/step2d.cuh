@@ -548,35 +548,35 @@ __device__ __forceinline__ void store_cell(const StepArgs& a, const PV& pv, cons
 template <class T, int K, int B, bool COMP, bool SQ, int NQ, int NM>
 __device__ __forceinline__ void row_update(T (&P)[NM], const T (&sx)[NM], const T (&V)[NM], const T (&FS)[NQ],
                                            const T (&un)[NM], T rx, T ry, T tdt) {
-    constexpr Tab2D<K, B> tb = make_tab2d<K, B>();
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
+    static_for<NM>([&](auto mc) {
+        constexpr int m = decltype(mc)::value;
         T sy = T(0);
-#pragma unroll
-        for (int p = 0; p < NQ; ++p)
-            if (tb.pS[p][m] != 0.0) sy = fma(FS[p], T(-tb.pS[p][m]), sy);
+        static_for<NQ>([&](auto pc) {
+            constexpr double w = Const2D<K, B>::tab.pS[decltype(pc)::value][m];
+            if constexpr (w != 0.0) sy = fma(FS[decltype(pc)::value], T(-w), sy);
+        });
         const T fsum = SQ ? fma(rx, sx[m] + sy, -V[m]) : fma(rx, sx[m], ry * sy) - V[m];
-        const T tc = tdt * T(tb.cm[m]);
+        constexpr double cm = Const2D<K, B>::tab.cm[m];
+        const T tc = tdt * T(cm);
         if constexpr (COMP) P[m] = -tc * fsum;
         else P[m] = fma(-tc, fsum, un[m]);
-    }
+    });
 }
 // ... and the north face: FN its flux (DEV: relative to the base of the row
 // above, gS moves it to this row's)
 template <class T, int K, int B, bool DEV, int NQ, int NM>
 __device__ __forceinline__ void add_north(T (&P)[NM], const T (&FN)[NQ], T gS, T ry, T tdt) {
-    constexpr Tab2D<K, B> tb = make_tab2d<K, B>();
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
+    static_for<NM>([&](auto mc) {
+        constexpr int m = decltype(mc)::value;
         T s = T(0);
-#pragma unroll
-        for (int p = 0; p < NQ; ++p)
-            if (tb.pN[p][m] != 0.0) s = fma(FN[p], T(tb.pN[p][m]), s);
-        if constexpr (DEV) {
-            if (tb.sN[m] != 0.0) s = fma(gS, T(-tb.sN[m]), s);
-        }
-        P[m] = fma(-(tdt * T(tb.cm[m])), ry * s, P[m]);
-    }
+        static_for<NQ>([&](auto pc) {
+            constexpr double w = Const2D<K, B>::tab.pN[decltype(pc)::value][m];
+            if constexpr (w != 0.0) s = fma(FN[decltype(pc)::value], T(w), s);
+        });
+        constexpr double sN = Const2D<K, B>::tab.sN[m], cm = Const2D<K, B>::tab.cm[m];
+        if constexpr (DEV && sN != 0.0) s = fma(gS, T(-sN), s);
+        P[m] = fma(-(tdt * T(cm)), ry * s, P[m]);
+    });
 }
 template <int NQ, int NV, class T>
 __device__ __forceinline__ void column(const T (&F)[NQ][NV], int v, T (&out)[NQ]) {

@@ -141,6 +141,15 @@ constexpr Tab2D<K, B> make_tab2d() {
     return t;
 }
 
+// The 2D table as a constant for device functions whose indices are constant
+// expressions (static_for): entries are immediates whatever the table's size.  A
+// local copy indexed in unrolled loops goes to each thread's stack where the
+// compiler does not fold it all, as it does not for Q^3 (12.7 KB).
+template <int K, int B>
+struct Const2D {
+    static constexpr Tab2D<K, B> tab = make_tab2d<K, B>();
+};
+
 // 1D tables for P^K with the (K+1)-point rule.
 template <int K>
 struct Tab1D {
