@@ -28,10 +28,14 @@ namespace crk {
 // equal the ones it evaluated last (uniform regions tie everywhere).  The
 // totals (FP64 sums) are formed where the caller reads them.  Measured (ncu): 0.158
 // -> 0.018 ms on that mesh, 0.075 -> 0.010 ms on 480 x 120.
-// relative bound, with margin, of the estimate's error: where speed_estimate
-// accepts a cell, p >= 1e-2 E bounds the cancellation in p (about 4 roundings
-// of E: 2.4e-5 of p, half of it in c), all else is a few roundings
+// relative bound, with margin, of the difference of two cells' errors: where
+// speed_estimate accepts a cell, E - KE >= 1e-2 E bounds the cancellation in p =
+// (gamma - 1)(E - KE), which takes about 9 roundings of E with those of an FP64
+// input (5.4e-7 E: 5.4e-5 of p, half of it in c), and p >= 1e-2 E, so gamma >=
+// 1.01, the rounding of gamma - 1; all else is a few roundings.  (p >= 1e-2 E
+// alone would let the cancellation grow with gamma - 1.)
 constexpr float SPEED_WINDOW = 1e-4f;
+constexpr float SPEED_CANCEL = 1e-2f;
 
 // FP64 wave speed of a cell's averages; status bits of a non-physical one
 template <int PHYS>
@@ -67,7 +71,7 @@ __device__ __forceinline__ bool speed_estimate(const float* av, float gamma, flo
     const float c = sqrtf(c2);
     s = (fabsf(w) + c) * rx;
     if (PHYS == PHYS_EULER) s += (fabsf(v) + c) * ry;
-    return av[0] > 1e-30f && E > 1e-30f && p > 1e-2f * E && c2 > 1e-30f && s > 1e-30f && s < 1e30f;
+    return av[0] > 1e-30f && E > 1e-30f && p > SPEED_CANCEL * fmaxf(1.f, gamma - 1.f) * E && c2 > 1e-30f && s > 1e-30f && s < 1e30f;
 }
 
 // block-wide maximum of an ordered key, sums and status bits; thread 0 holds the results
