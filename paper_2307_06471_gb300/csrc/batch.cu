@@ -677,37 +677,40 @@ int crkdg_batch_autotune(crkdg_batch* b, double cfl, double* best_us) {
     BCK(cudaStreamSynchronize(b->stream));
     BCK(cudaMemcpy(st.data(), b->d_states, b->n * sizeof(DevState), cudaMemcpyDeviceToHost));
     BCK(cudaMemcpy(cu.data(), b->d_curs, b->n * sizeof(int), cudaMemcpyDeviceToHost));
-    const int rows[] = {8, 16, 32, 64};
-    const int wpbs[] = {2, 4, 8};
+    // candidates: the current shape first (tuning never makes it worse), then a
+    // ladder over the lengths default_shape may choose and longer ones
+    std::vector<std::pair<int, int>> cand{{b->seg_rows, b->wpb}};
+    for (int L : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 64})
+        for (int w : {2, 4, 8})
+            if (std::make_pair(L, w) != cand[0]) cand.emplace_back(L, w);
     cudaEvent_t e0, e1;
     BCK(cudaEventCreate(&e0));
     BCK(cudaEventCreate(&e1));
     double best = 1e30;
     int bl = b->seg_rows, bw = b->wpb;
-    for (int L : rows)
-        for (int w : wpbs) {
-            if (crkdg_batch_set_launch(b, L, w) != CRKDG_OK) continue;
-            float t[4];
-            for (int it = 0; it < 4; ++it) {
-                BCK(cudaMemcpy(b->d_states, st.data(), b->n * sizeof(DevState), cudaMemcpyHostToDevice));
-                BCK(cudaMemcpy(b->d_curs, cu.data(), b->n * sizeof(int), cudaMemcpyHostToDevice));
-                int rs = start_run(b, cfl, 1e30);
-                if (rs) return rs;
-                BCK(cudaEventRecord(e0, b->stream));
-                int r = enqueue_batch_step(b, b->pending, b->M_pending, b->pp_pending);
-                if (r) return r;
-                BCK(cudaEventRecord(e1, b->stream));
-                BCK(cudaEventSynchronize(e1));
-                BCK(cudaEventElapsedTime(&t[it], e0, e1));
-            }
-            std::sort(t + 1, t + 4);
-            const double us = 1000.0 * t[2];
-            if (us < best) {
-                best = us;
-                bl = L;
-                bw = w;
-            }
+    for (const auto& c : cand) {
+        if (crkdg_batch_set_launch(b, c.first, c.second) != CRKDG_OK) continue;
+        float t[4];
+        for (int it = 0; it < 4; ++it) {
+            BCK(cudaMemcpy(b->d_states, st.data(), b->n * sizeof(DevState), cudaMemcpyHostToDevice));
+            BCK(cudaMemcpy(b->d_curs, cu.data(), b->n * sizeof(int), cudaMemcpyHostToDevice));
+            int rs = start_run(b, cfl, 1e30);
+            if (rs) return rs;
+            BCK(cudaEventRecord(e0, b->stream));
+            int r = enqueue_batch_step(b, b->pending, b->M_pending, b->pp_pending);
+            if (r) return r;
+            BCK(cudaEventRecord(e1, b->stream));
+            BCK(cudaEventSynchronize(e1));
+            BCK(cudaEventElapsedTime(&t[it], e0, e1));
         }
+        std::sort(t + 1, t + 4);
+        const double us = 1000.0 * t[2];
+        if (us < best) {
+            best = us;
+            bl = c.first;
+            bw = c.second;
+        }
+    }
     BCK(cudaMemcpy(b->d_states, st.data(), b->n * sizeof(DevState), cudaMemcpyHostToDevice));
     BCK(cudaMemcpy(b->d_curs, cu.data(), b->n * sizeof(int), cudaMemcpyHostToDevice));
     cudaEventDestroy(e0);
