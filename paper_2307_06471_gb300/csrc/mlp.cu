@@ -444,6 +444,25 @@ bool grow(V*& p, size_t& cap, size_t n) {
     return true;
 }
 
+// A host buffer that a copy on a stream may still be reading: the copy is done
+// once wait() has returned, and before the guard goes.  (Copies from pageable
+// memory may return before they have read it where the GPU reads pageable
+// memory itself, as it does beside a Grace host.)
+struct CopyGuard {
+    cudaEvent_t done = nullptr;
+    ~CopyGuard() {
+        if (!done) return;
+        cudaEventSynchronize(done);
+        cudaEventDestroy(done);
+    }
+    cudaError_t copy(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+        cudaError_t e = done ? cudaSuccess : cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+        return e == cudaSuccess ? cudaEventRecord(done, st) : e;
+    }
+    cudaError_t wait() { return done ? cudaEventSynchronize(done) : cudaSuccess; }
+};
+
 double uniform01(uint64_t& s) { return ((splitmix(s) >> 11) + 0.5) * (1.0 / 9007199254740992.0); }
 
 }  // namespace
@@ -599,13 +618,15 @@ int crkdg_mlp_train(crkdg_mlp* m, const float* X_dev, const float* y_dev, int n,
     if (!grow(m->d_idx, m->idx_cap, n)) return mfail(CRKDG_ENOMEM, "cudaMalloc failed");
     std::vector<int> perm(n);
     for (int i = 0; i < n; ++i) perm[i] = i;
+    CopyGuard guard;   // of perm (destroyed before it)
     uint64_t s = seed;
     for (int ep = 0; ep < epochs; ++ep) {
+        MCK(guard.wait());   // the last epoch's order has left; its minibatches run on
         for (int i = n - 1; i > 0; --i) {   // Fisher--Yates shuffle
             const int j = (int)(splitmix(s) % (uint64_t)(i + 1));
             std::swap(perm[i], perm[j]);
         }
-        MCK(cudaMemcpyAsync(m->d_idx, perm.data(), n * sizeof(int), cudaMemcpyHostToDevice, m->stream));
+        MCK(guard.copy(m->d_idx, perm.data(), n * sizeof(int), m->stream));
         for (int b = 0; b < nb; ++b) {
             const int b0 = b * batch, nbatch = std::min(batch, n - b0);
             m->adam_t += 1;
