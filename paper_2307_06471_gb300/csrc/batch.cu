@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -108,6 +109,7 @@ struct crkdg_batch {
     double* d_tab = nullptr;
     double* d_stage = nullptr;             // get_state's staging, as large as the largest problem read
     size_t stage_cap = 0;
+    std::mutex stage;                      // one call at a time has it
     unsigned long long* d_flags = nullptr;
     cudaStream_t stream = nullptr;
     int seg_rows = 32, wpb = 4;            // default_shape, crkdg_batch_set_launch
@@ -486,6 +488,7 @@ int crkdg_batch_set_state(crkdg_batch* b, int p, const double* h, double t) {
 
 int crkdg_batch_get_state(crkdg_batch* b, int p, double* h) {
     if (!b || !h || p < 0 || p >= b->n) return bfail(CRKDG_EINVAL, "bad argument");
+    std::lock_guard<std::mutex> own(b->stage);
     int cur = 0;
     int r = get_cur(b, p, &cur);
     if (r) return r;

@@ -476,7 +476,8 @@ struct crkdg_mlp {
     cudaStream_t stream = nullptr;
     long long adam_t = 0;
     // training workspace, kept between calls: the blocks' gradients and loss
-    // sums, the shuffled rows, the minibatches' losses
+    // sums, the shuffled rows, the minibatches' losses; one call at a time has it
+    std::mutex work;
     float* d_gpart = nullptr;
     float* d_lpart = nullptr;
     int* d_idx = nullptr;
@@ -597,6 +598,7 @@ static cudaError_t enqueue_grad(crkdg_mlp* m, const float* X, const float* y, co
 int crkdg_mlp_loss_grad(crkdg_mlp* m, const float* X_dev, const float* y_dev, int n, double pos_weight, double* loss,
                         float* grad_host) {
     if (!m || !X_dev || !y_dev || n < 1) return mfail(CRKDG_EINVAL, "bad argument");
+    std::lock_guard<std::mutex> own(m->work);
     int r = train_workspace(m, n, 1);
     if (r) return r;
     MCK(enqueue_grad(m, X_dev, y_dev, nullptr, n, pos_weight, m->d_loss, AdamArgs{}, false));
@@ -612,6 +614,7 @@ int crkdg_mlp_train(crkdg_mlp* m, const float* X_dev, const float* y_dev, int n,
                     double pos_weight, unsigned long long seed, double* last_epoch_loss) {
     if (!m || !X_dev || !y_dev || n < 1 || epochs < 0 || batch < 1 || !(lr > 0.0))
         return mfail(CRKDG_EINVAL, "bad argument");
+    std::lock_guard<std::mutex> own(m->work);
     const int nb = (int)(((long long)n + batch - 1) / batch);   // minibatches of an epoch
     int r = train_workspace(m, std::min(n, batch), nb);
     if (r) return r;
