@@ -560,7 +560,8 @@ static int train_blocks(int n) {
     return (int)std::min<long long>(((long long)n + TILE - 1) / TILE, 2LL * std::max(1, crk::sm_count()));
 }
 
-// workspace for gradients over up to n samples and `losses` minibatch losses
+// workspace for gradients over up to n samples and `losses` minibatch losses,
+// and the kernel's shared memory
 static int train_workspace(crkdg_mlp* m, int n, size_t losses) {
     const size_t blocks = train_blocks(n);
     if (blocks > m->part_blocks) {
@@ -571,6 +572,9 @@ static int train_workspace(crkdg_mlp* m, int n, size_t losses) {
         m->part_blocks = blocks;
     }
     if (!grow(m->d_loss, m->loss_cap, losses)) return mfail(CRKDG_ENOMEM, "cudaMalloc failed");
+    // an attribute of the kernel on the current device: set by every call, which
+    // may be the device's first
+    MCK(cudaFuncSetAttribute(mlp_fwdbwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)));
     return CRKDG_OK;
 }
 
@@ -580,13 +584,6 @@ static int train_workspace(crkdg_mlp* m, int n, size_t losses) {
 // idx are read before it has completed).
 static cudaError_t enqueue_grad(crkdg_mlp* m, const float* X, const float* y, const int* idx, int n, double pw,
                                 double* loss, const AdamArgs& ad, bool follows) {
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [&] {
-        attr_err = cudaFuncSetAttribute(mlp_fwdbwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)sizeof(TrainSmem));
-    });
-    if (attr_err != cudaSuccess) return attr_err;
     const int nb = train_blocks(n);
     const cudaError_t e = launch(&mlp_fwdbwd_kernel, nb, TRAIN_THREADS, sizeof(TrainSmem), follows, m->stream, m->d_prm, X, y,
                                  idx, n, (float)pw, m->d_gpart, m->d_lpart);
@@ -656,21 +653,12 @@ int crkdg_mlp_predict(crkdg_mlp* m, const float* X_dev, int n, float* logits_dev
     if (!m || !X_dev || !logits_dev || n < 1) return mfail(CRKDG_EINVAL, "bad argument");
     const size_t smem =
         sizeof(crk::MlpSmem) + (PREDICT_THREADS / 32) * (32 * crk::MLP_INP + 64) * sizeof(__nv_bfloat16);
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    static int per_sm = 1;
-    std::call_once(once, [&] {
-        for (auto k : {mlp_predict_kernel<true>, mlp_predict_kernel<false>})
-            if (attr_err == cudaSuccess)
-                attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (attr_err == cudaSuccess)
-            attr_err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_predict_kernel<true>,
-                                                                     PREDICT_THREADS, smem);
-    });
-    MCK(attr_err);
+    auto kern = reinterpret_cast<uintptr_t>(X_dev) % 8 == 0 ? mlp_predict_kernel<true> : mlp_predict_kernel<false>;
+    int per_sm = 1;   // (of the current device, as the attribute is)
+    MCK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PREDICT_THREADS, smem));
     const long long tiles = ((long long)n + PREDICT_THREADS - 1) / PREDICT_THREADS;
     const int grid = (int)std::min<long long>(tiles, (long long)std::max(1, per_sm) * std::max(1, crk::sm_count()));
-    auto kern = reinterpret_cast<uintptr_t>(X_dev) % 8 == 0 ? mlp_predict_kernel<true> : mlp_predict_kernel<false>;
     kern<<<grid, PREDICT_THREADS, smem, m->stream>>>(m->d_prm, X_dev, n, logits_dev);
     MCK(cudaGetLastError());
     MCK(cudaStreamSynchronize(m->stream));
