@@ -312,6 +312,21 @@ int get_cur(const crkdg_batch* b, int p, int* cur) {
     return CRKDG_OK;
 }
 
+// get_state's staging buffer holds at least n values
+bool stage_room(crkdg_batch* b, size_t n) {
+    if (n <= b->stage_cap) return true;
+    if (b->d_stage) cudaFree(b->d_stage);
+    b->d_stage = nullptr;
+    b->stage_cap = 0;
+    if (cudaMalloc(&b->d_stage, n * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        b->d_stage = nullptr;
+        return false;
+    }
+    b->stage_cap = n;
+    return true;
+}
+
 StepArgs problem_args(const crkdg_batch* b, int p) {
     StepArgs a = batch_args(b);
     const BatchProblem& pb = b->probs[p];
@@ -497,23 +512,15 @@ int crkdg_batch_get_state(crkdg_batch* b, int p, double* h) {
     const char* base = static_cast<char*>(b->buf[cur]) + pb.offset * b->esize;
     const bool f32 = b->precision == CRKDG_F32;
     // the copy a pending limiter is applied to, and the FP64 values of an FP32
-    // state: in the batch's staging buffer, kept between calls (FP64 first)
-    const size_t limited = b->pending ? (n * b->esize + 7) / 8 : 0, need = (f32 ? n : 0) + limited;
-    if (need > b->stage_cap) {
-        if (b->d_stage) cudaFree(b->d_stage);
-        b->d_stage = nullptr;
-        b->stage_cap = 0;
-        if (cudaMalloc(&b->d_stage, need * sizeof(double)) != cudaSuccess) {
-            cudaGetLastError();
-            b->d_stage = nullptr;
-            return bfail(CRKDG_ENOMEM, "cudaMalloc failed");
-        }
-        b->stage_cap = need;
-    }
+    // state: in the batch's staging buffer, kept between calls (FP64 first).
+    // Where the device has no room for the values, they are widened on the host.
+    const size_t limited = b->pending ? (n * b->esize + 7) / 8 : 0;
+    const bool widen = f32 && stage_room(b, n + limited);
+    if (!widen && !stage_room(b, limited)) return bfail(CRKDG_ENOMEM, "cudaMalloc of the limited copy failed");
     const void* src = base;
     if (b->pending) {
         // the stored state is pending the limiter of its last step: apply it to a copy
-        void* tmp = b->d_stage + (f32 ? n : 0);
+        void* tmp = b->d_stage + (widen ? n : 0);
         BCK(cudaMemcpyAsync(tmp, base, n * b->esize, cudaMemcpyDeviceToDevice, b->stream));
         StepArgs a = problem_args(b, p);
         a.ds = b->d_states + p;
@@ -522,6 +529,13 @@ int crkdg_batch_get_state(crkdg_batch* b, int p, double* h) {
         a.pp_eps = b->pp_pending;
         BCK(crk::launch_limit2d(crk::PHYS_EULER, b->precision, b->k, b->basis, a, tmp, b->d_flags, b->stream));
         src = tmp;
+    }
+    if (f32 && !widen) {
+        std::vector<float> f(n);
+        BCK(cudaMemcpyAsync(f.data(), src, n * 4, cudaMemcpyDeviceToHost, b->stream));
+        BCK(cudaStreamSynchronize(b->stream));
+        for (size_t i = 0; i < n; ++i) h[i] = f[i];
+        return CRKDG_OK;
     }
     if (f32) {   // widened on the GPU
         BCK(crk::launch_f32_to_f64(static_cast<const float*>(src), b->d_stage, n, 0, b->stream));
