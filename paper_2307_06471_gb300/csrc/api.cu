@@ -1015,7 +1015,7 @@ int crkdg_run_fixed(crkdg_ctx* c, int n_steps, double dt) {
     CK(crk::launch_step1d(c->kphys, c->precision, c->k, a, n_steps, (warps + blocks - 1) / blocks * 32, blocks,
                           c->stream));
     if (n_steps % 2) c->cur ^= 1;
-    c->t += n_steps * dt;
+    for (int i = 0; i < n_steps; ++i) c->t += dt;   // as the run's stage times and a stepping caller's do
     return CRKDG_OK;
 }
 
