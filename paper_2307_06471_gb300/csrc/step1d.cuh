@@ -184,7 +184,9 @@ __device__ __forceinline__ void step1d_linear(const StepArgs& a, const Line& ln,
     }
     T west = shfl_up(tR, 1), east = shfl_down(tL, 1);
     // exterior trace at a boundary on the inflow side, sum_i b_i of the stages'
+    // (in: that sum of the interior traces)
     auto exterior = [&](const BCSide& bc, T in, double xb) {
+        if (bc.type == BC_OUTFLOW) return in;
         T e = T(0);
         for (int i = 0; i < S; ++i) {
             const T bi = tab_bT<T>(a, i);

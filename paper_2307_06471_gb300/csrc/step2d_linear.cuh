@@ -187,8 +187,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
             out[m] = acc;
         });
     };
-    // exterior trace at a non-periodic side: m * interior + constant state, or
-    // the side's data at its face `face`
+    // exterior trace, sum_i b_i of the stages', at a non-periodic side: m *
+    // interior + the constant state's share, or the side's data at its face `face`
     auto bc_trace = [&](int side, int face, const T* in, T* out) {
         const BCSide& b = a.bc[side];
         if (DATA && !b.affine) {
@@ -197,7 +197,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? CRK_LIN_MINB : 1) step2d
             for (int q = 0; q < NT; ++q) out[q] = d[q];
             return;
         }
-        const T c = sizeof(T) == 4 ? T(b.cf[0]) : T(b.cd[0]);
+        // lin_gamma[0] = sum_i b_i
+        const T c = sizeof(T) == 4 ? T(a.lin_gammaf[0]) * T(b.cf[0]) : T(a.lin_gamma[0]) * T(b.cd[0]);
 #pragma unroll
         for (int q = 0; q < NT; ++q) out[q] = T(b.m[0]) * in[q] + (q == 0 ? c : T(0));
     };
