@@ -1211,7 +1211,14 @@ int crkdg_get_limit_mode(const crkdg_ctx* c, int* mode) {
 
 int crkdg_get_launch(const crkdg_ctx* c, int* seg_rows, int* wpb) {
     if (check_ctx(c)) return CRKDG_EINVAL;
-    if (seg_rows) *seg_rows = c->seg_rows;
+    if (seg_rows) {
+        *seg_rows = c->seg_rows;
+        if (c->dim == 2) {   // longer where the room of the seam scratch leaves fewer segments
+            int ns, nseg;
+            step_segs(c, &ns, &nseg);
+            *seg_rows = std::max(c->seg_rows, (c->mesh.ny + nseg - 1) / nseg);
+        }
+    }
     if (wpb) *wpb = c->wpb;
     return CRKDG_OK;
 }
