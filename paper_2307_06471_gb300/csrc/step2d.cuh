@@ -481,11 +481,14 @@ __device__ __forceinline__ T new_speed(const StepArgs& a, const PV& pv, const T*
     }
 }
 
-// hi' + lo' = hi + lo + inc at element ix of a compensated state (TwoSum)
+// hi' + lo' = hi + lo + inc at element ix of a compensated state (TwoSum).  u^n
+// is read through the read-only path: as ordinary loads the modes' hi and lo
+// waited for one another's stores (the compiler does not see across this
+// function that uout is another buffer), 72 round trips a row for Q^2.
 template <class T>
 __device__ __forceinline__ void store_comp(const T* __restrict__ uin, T* __restrict__ uout, size_t ix, size_t lo_off,
                                            T inc, T& hi_out, T& lo_out) {
-    const T hi = uin[ix], lo = uin[lo_off + ix];
+    const T hi = __ldg(uin + ix), lo = __ldg(uin + lo_off + ix);
     const T d = inc + lo;
     const T sum = hi + d;
     const T bv = sum - hi;
