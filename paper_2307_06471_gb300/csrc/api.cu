@@ -1009,9 +1009,7 @@ int crkdg_run_fixed(crkdg_ctx* c, int n_steps, double dt) {
     a.t = c->t;
     a.dt = dt;
     set_linear(c, a);
-    // a power of two of blocks, up to 8, for a warp each where that reaches
-    int blocks = 1;
-    while (blocks < 8 && blocks < warps) blocks *= 2;
+    const int blocks = crk::run1d_blocks(warps, c->esize);
     CK(crk::launch_step1d(c->kphys, c->precision, c->k, a, n_steps, (warps + blocks - 1) / blocks * 32, blocks,
                           c->stream));
     if (n_steps % 2) c->cur ^= 1;

@@ -9,10 +9,10 @@
 namespace crk {
 namespace {
 
-template <class T, int K, int PHYS>
-cudaError_t run_step1d(const StepArgs& a, int n_steps, int threads, int blocks, cudaStream_t st) {
+template <class T, int K, int PHYS, bool ONE>
+cudaError_t run_step1d_t(const StepArgs& b, int n_steps, int threads, int blocks, cudaStream_t st) {
     constexpr int NDOF = Phys<T, PHYS>::NV * (K + 1);
-    auto kern = step1d_kernel<T, K, PHYS>;
+    auto kern = step1d_kernel<T, K, PHYS, ONE>;
     static std::once_flag once;
     static cudaError_t attr_err = cudaSuccess;
     std::call_once(once, [&] {
@@ -23,10 +23,8 @@ cudaError_t run_step1d(const StepArgs& a, int n_steps, int threads, int blocks, 
                                             227 * 1024 - (int)fa.sharedSizeBytes);
     });
     if (attr_err != cudaSuccess) return attr_err;
-    const size_t smem = (size_t)(a.s > 1 ? a.s - 1 : 1) * NDOF * sizeof(T) * threads;
-    StepArgs b = a;
-    set_derived(b);
-    if (n_steps == 1) {
+    const size_t smem = (size_t)(b.s > 1 ? b.s - 1 : 1) * NDOF * sizeof(T) * threads;
+    if constexpr (ONE) {
         kern<<<blocks, threads, smem, st>>>(b, n_steps);
         return cudaGetLastError();
     }
@@ -45,10 +43,18 @@ cudaError_t run_step1d(const StepArgs& a, int n_steps, int threads, int blocks, 
 }
 
 template <class T, int K, int PHYS>
+cudaError_t run_step1d(const StepArgs& a, int n_steps, int threads, int blocks, cudaStream_t st) {
+    StepArgs b = a;
+    set_derived(b);
+    return n_steps == 1 || blocks == 1 ? run_step1d_t<T, K, PHYS, true>(b, n_steps, threads, blocks, st)
+                                       : run_step1d_t<T, K, PHYS, false>(b, n_steps, threads, blocks, st);
+}
+
+template <class T, int K, int PHYS>
 cudaError_t run_info1d(int s, KernelInfo* info) {
     constexpr int NDOF = Phys<T, PHYS>::NV * (K + 1);
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, step1d_kernel<T, K, PHYS>);
+    cudaError_t e = cudaFuncGetAttributes(&fa, step1d_kernel<T, K, PHYS, true>);
     if (e != cudaSuccess) return e;
     info->regs = fa.numRegs;
     info->max_threads = fa.maxThreadsPerBlock;

@@ -38,7 +38,19 @@ cudaError_t launch_limit2d(int phys, int prec, int k, int basis, const StepArgs&
 // projection of point values (device FP64 [cell][q][v])
 cudaError_t launch_project(int dim, int phys, int prec, int k, int basis, const double* vals, void* u, int ncell,
                            cudaStream_t st);
-// 1D fused step; n_steps > 1 requires one block
+// Blocks (of one cluster) of a 1D run of `warps` warps, up to 32: a power of two, up
+// to the portable cluster size, for a warp each where that reaches.  A few warps
+// stay in one block, whose barrier costs a microsecond less than a cluster's: in
+// FP64 as many as the SM's FP64 pipe takes without a queue (a step of Euler P^2,
+// one block / cluster: 2 warps 22.3 / 23.2 us, 3 warps 22.4 / 23.3, 4 warps 24.6 /
+// 23.2), in FP32 those of a block (4 warps 1.51 / 2.36).
+inline int run1d_blocks(int warps, size_t esize) {
+    int blocks = 1;
+    if (warps > (esize == 4 ? 4 : 3))
+        while (blocks < 8 && blocks < warps) blocks *= 2;
+    return blocks;
+}
+// 1D fused step; n_steps > 1: a run, its blocks are one cluster
 cudaError_t launch_step1d(int phys, int prec, int k, const StepArgs& a, int n_steps, int threads, int blocks,
                           cudaStream_t st);
 cudaError_t info_step1d(int phys, int prec, int k, int s, KernelInfo* info);

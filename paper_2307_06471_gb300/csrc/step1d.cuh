@@ -10,7 +10,8 @@
 // of the Legendre derivative, the upwind jump on the inflow face, no point
 // values -- 35 instead of 190 FP64 operations a cell for P^2.  A step is bound
 // by its FP64 operations where warps share an SM's FP64 pipe and by the
-// dependent chain otherwise, so a run spreads its warps over up to 8 SMs.  160
+// dependent chain otherwise, so a run spreads its warps over up to 8 SMs (a few
+// warps do with one SM, and without the cluster's barrier: run1d_blocks).  160
 // cells, P^2, SSP-RK3, FP64, 160 steps: 1.33 ms in one block and quadrature form,
 // 0.35 ms so.
 #pragma once
@@ -20,8 +21,8 @@
 
 namespace crk {
 
-// Most blocks of a run (the portable cluster size) and its most warps per block
-constexpr int RUN1D_BLOCKS = 8, RUN1D_WARPS = 4;
+// Most warps per block of a run (launch.h: run1d_blocks)
+constexpr int RUN1D_WARPS = 4;
 
 // What a lane needs of the mesh
 struct Line {
@@ -35,7 +36,7 @@ __device__ __forceinline__ void step1d_cell(const StepArgs& a, const Line& ln, c
                                             double dt, T rx, const Slot& slot, const T (&un)[NV][NM], T (&out)[NV][NM]) {
     constexpr Tab1D<K> tb = make_tab1d<K>();
     constexpr int NQ = K + 1, NDOF = NV * NM;
-    const T tdt = T(dt);
+    const T tdt = opaque(T(dt));
     const int S = a.s;
     T V[NV][NM], FR[NV];
 #pragma unroll
@@ -45,20 +46,18 @@ __device__ __forceinline__ void step1d_cell(const StepArgs& a, const Line& ln, c
         for (int m = 0; m < NM; ++m) V[v][m] = T(0);
     }
     for (int i = 0; i < S; ++i) {
-        const double bid = tab_b(a, i);
-        const T bi = T(bid);
+        const T bi = tab_bT<T>(a, i);
         const bool need_L = i < S - 1;
-        if (!need_L && bid == 0.0) continue;
-        const double ti = t0 + tab_c(a, i) * dt;
+        if (!need_L && bi == T(0)) continue;
         T w[NV][NM];
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
             for (int m = 0; m < NM; ++m) w[v][m] = un[v][m];
         for (int j = 0; j < i; ++j) {
-            const double ad = tab_a(a, i, j);
-            if (ad == 0.0) continue;
-            const T aij = T(ad) * tdt;
+            const T ad = tab_aT<T>(a, i, j);
+            if (ad == T(0)) continue;
+            const T aij = ad * tdt;
 #pragma unroll
             for (int v = 0; v < NV; ++v)
 #pragma unroll
@@ -110,7 +109,7 @@ __device__ __forceinline__ void step1d_cell(const StepArgs& a, const Line& ln, c
                     slot(i * NDOF + v * NM + m) =
                         T(tb.cm[m]) * (rx * (fr[v] * T(tb.tR[m]) - fl[v] * T(tb.tL[m])) - vol[v][m]);
         }
-        if (bid == 0.0) continue;
+        if (bi == T(0)) continue;
 #pragma unroll
         for (int v = 0; v < NV; ++v)
 #pragma unroll
@@ -118,11 +117,24 @@ __device__ __forceinline__ void step1d_cell(const StepArgs& a, const Line& ln, c
         T tLn[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) tLn[v] = shfl_down(tL[v], 1);
-        if (ln.bcW && ln.lane == 0)
-            bc_exterior<T, NV>(a.bc[0], 0, tLn, [&](double& x, double& y, double& t) { x = a.x0; y = 0.0; t = ti; }, tR);
-        if (ln.bcE && ln.col == ln.nx - 1)
-            bc_exterior<T, NV>(a.bc[1], 0, tR, [&](double& x, double& y, double& t) { x = a.x0 + ln.nx * a.dx; y = 0.0; t = ti; },
-                               tLn);
+        if (ln.bcW && ln.lane == 0) {
+            cold_branch();
+            const int ic = opaque(i);
+            bc_exterior<T, NV>(a.bc[0], 0, tLn, [&](double& x, double& y, double& t) {
+                x = a.x0;
+                y = 0.0;
+                t = t0 + tab_c(a, ic) * dt;
+            }, tR);
+        }
+        if (ln.bcE && ln.col == ln.nx - 1) {
+            cold_branch();
+            const int ic = opaque(i);
+            bc_exterior<T, NV>(a.bc[1], 0, tR, [&](double& x, double& y, double& t) {
+                x = a.x0 + ln.nx * a.dx;
+                y = 0.0;
+                t = t0 + tab_c(a, ic) * dt;
+            }, tLn);
+        }
         T F[NV];
         llf<T, PHYS, 0>(ph, tR, tLn, F);
 #pragma unroll
@@ -213,7 +225,9 @@ __device__ __forceinline__ void step1d_linear(const StepArgs& a, const Line& ln,
     }
 }
 
-template <class T, int K, int PHYS>
+// ONE: a single step, or a run of one block, whose warps meet at the block's
+// barrier; otherwise a run of one cluster
+template <class T, int K, int PHYS, bool ONE>
 __global__ void __launch_bounds__(256) step1d_kernel(const StepArgs a, int n_steps) {
     constexpr int NM = K + 1, NV = Phys<T, PHYS>::NV, NDOF = NV * NM;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -242,15 +256,16 @@ __global__ void __launch_bounds__(256) step1d_kernel(const StepArgs a, int n_ste
         ph.bx = T(a.beta[0]);
         ph.by = T(0);
     } else {
-        ph.gamma = T(a.gamma);
-        ph.gm1 = T(a.gamma - 1.0);
+        // (held in registers: formed again at every use they are FP64 arithmetic)
+        ph.gamma = opaque(T(a.gamma));
+        ph.gm1 = opaque(T(a.gamma - 1.0));
     }
     const T rx = sizeof(T) == 4 ? T(a.rxf) : T(a.rx);
     const T* src = static_cast<const T*>(a.uin);
     const auto cluster = cooperative_groups::this_cluster();
     // a block's shared memory may be written once the block has started: every
     // block says so here, and the first push waits for all of them
-    if (n_steps > 1) cluster.barrier_arrive();
+    if constexpr (!ONE) cluster.barrier_arrive();
     T un[NV][NM], out[NV][NM];
 #pragma unroll
     for (int v = 0; v < NV; ++v)
@@ -266,9 +281,12 @@ __global__ void __launch_bounds__(256) step1d_kernel(const StepArgs a, int n_ste
             else step1d_cell<T, K, PHYS, NV, NM>(a, ln, ph, t0, a.dt, rx, slot, un, out);
         }
         if (step + 1 == n_steps) break;
-        if (step == 0) cluster.barrier_wait();
+        if constexpr (!ONE)
+            if (step == 0) cluster.barrier_wait();
         auto push = [&](int warp, int side) {   // to a warp's halo lane
-            T* h = cluster.map_shared_rank(&halo[step & 1][warp % wpb][side][0], warp / wpb);
+            T* h;
+            if constexpr (ONE) h = &halo[step & 1][warp][side][0];
+            else h = cluster.map_shared_rank(&halo[step & 1][warp % wpb][side][0], warp / wpb);
 #pragma unroll
             for (int v = 0; v < NV; ++v)
 #pragma unroll
@@ -276,7 +294,8 @@ __global__ void __launch_bounds__(256) step1d_kernel(const StepArgs a, int n_ste
         };
         if (lane == 1 && n_out > 0 && (ln.per || gw > 0)) push(gl, 1);
         if (lane == n_out && n_out > 0 && (ln.per || gw + 1 < warps)) push(gr, 0);
-        cluster.sync();
+        if constexpr (ONE) __syncthreads();
+        else cluster.sync();
         const bool hw = lane == 0 && !ln.bcW, he = lane == n_out + 1 && !ln.bcE;
 #pragma unroll
         for (int v = 0; v < NV; ++v)
