@@ -145,10 +145,12 @@ size_t seam_seg_bytes(const crkdg_ctx* c, bool fused) {
 // whether the quadrature step leaves the faces between its segments to the
 // seam launches (the compensated state without
 // deviation fluxes recomputes halo rows)
-bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load) {
-    return c->precision != CRKDG_F32C && !c->seams_off && crk::use_seams(c->esize, c->tab.s, c->nm, c->precision == CRKDG_F32D, lim_on_load,
-                                                             c->mesh.ny, nseg);
+bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load, int stages) {
+    return c->precision != CRKDG_F32C && !c->seams_off &&
+           crk::use_seams(c->esize, stages, c->nm, c->k + 1, c->nv, c->precision == CRKDG_F32D, lim_on_load, c->mesh.ny, nseg,
+                          (long long)((c->mesh.nx + 29) / 30) * nseg, std::max(1, crk::sm_count()));
 }
+bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load) { return step_seams(c, nseg, lim_on_load, c->tab.s); }
 
 // launch geometry of the quadrature step (its scratch bounds the segments)
 void step_segs(const crkdg_ctx* c, bool fused, int* ns, int* nseg) {
@@ -916,7 +918,7 @@ static int enqueue_fe(crkdg_ctx* c, const void* in, void* out, double t, double 
     if (r) return r;
     a.partials = c->d_partials;
     a.seam = c->d_seam;
-    a.seams = step_seams(c, nseg, false);
+    a.seams = step_seams(c, nseg, false, 1);
     CK(crk::launch_step2d(c->kphys, c->precision, c->k, c->basis, a, c->wpb, c->stream));
     return CRKDG_OK;
 }

@@ -202,7 +202,10 @@ int upload(V*& d, const std::vector<V>& h) {
 // batch whose tables could not be made runs nothing until they are.
 int build_tables(crkdg_batch* b) {
     free_tables(b);
-    bool seams = crk::use_seams(b->esize, b->tab.s, b->nm, false, false, b->seg_rows, 1);
+    long long warps = 0;
+    for (const auto& pb : b->probs) warps += (long long)((pb.nx + 29) / 30) * ((pb.ny + b->seg_rows - 1) / b->seg_rows);
+    bool seams = crk::use_seams(b->esize, b->tab.s, b->nm, b->k + 1, b->nv, false, false, b->seg_rows, 1, warps,
+                                std::max(1, crk::sm_count()));
     size_t room = crk::seam_room(b->elems * b->esize);
     long long slots = 0;
     for (;;) {

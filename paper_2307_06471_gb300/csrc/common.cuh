@@ -396,23 +396,47 @@ inline int seam_flux_blocks(size_t esize, int nq, int nx, int n_segs) {
     return (int)((n + t - 1) / t);
 }
 // Whether a step whose segments have ny / n_segs rows leaves its seams to the
-// seam launches instead of recomputing the row beyond each end of a segment.
+// seam launches instead of recomputing the row beyond each end of a segment;
+// warps: the step's, sms: the device's SMs.
 // FP64 always: its pipe is the bound, and a recomputed row costs what any row
 // does (P^2 SSP-RK3 on 640 x 160, 3 rows a segment: 1.40 ms with halo rows, 0.99
-// with seams; Q^2 RK4 on 80 x 80, 1 row: 0.70 and 0.26 ms).  FP32: the seam
-// launches and their traffic cost about 0.02 ms, so it depends on what a row
-// costs (stages x modes) and on the rows of a segment.  Q^2 RK4 (36) on 1001 x
-// 613, ms per 4 steps with halo rows / seams: 1 row 2.28 / 1.66, 3 rows 1.39 /
-// 1.29, 6 rows 1.17 / 1.13; in the deviation form on 320 x 320, 20 steps, 3
-// rows 1.99 / 1.80, 6 rows 2.92 / 2.60.  P^2 SSP-RK3 (18) on 1920 x 480: 1 row
-// 2.28 / 1.72, 2 rows 1.58 / 1.62, 4 rows 1.23 / 1.29.  P^1 SSP-RK3 (9) on 480 x
-// 120, 2 rows, one step: 0.062 / 0.072.
-// Deviation form (dev), ms with halo rows / seams: 640^2, 12 rows, 6 steps 1.95 /
-// 1.89; 1280^2, 46 rows, 3 steps 3.59 / 3.37.
-inline bool use_seams(size_t esize, int stages, int modes, bool dev, bool lim_on_load, int ny, int n_segs) {
+// with seams; Q^2 RK4 on 80 x 80, 1 row: 0.70 and 0.26 ms).
+// FP32: the seam launches and their traffic cost what they cost, so it depends on
+// what a row costs (stages x modes x points) and on the rows of a segment.  Times
+// with seams over times with halo rows, in the default launch shapes (one wave
+// of warps) of n x n meshes, graph replays of 16 steps (k = 2 row cost 378 for P^2
+// SSP-RK3, 504 RK4, 567 for Q^2 SSP-RK3, 756 RK4; k = 3 from 960):
+//   n               64    128    256    320    400    512    800   1280
+//   rows             1      1      2      3      5      8     18     46
+//   P^2 SSP-RK3   1.09   1.05   1.21   1.16   1.14   1.10   1.09   1.05
+//   P^2 RK4       1.00   0.95   1.10   1.07   1.07   1.06   1.06   1.03
+//   Q^2 SSP-RK3   1.00   0.90   1.04   1.06   1.02   1.05   1.07   1.04
+//   Q^2 RK4       0.89   0.81   0.95   0.98   0.98   1.01   1.02   1.00
+//   P^3 SSP-RK3   0.74   0.70   0.82   0.85   0.90   0.97   0.97   0.98
+// deviation form (dev):
+//   P^2 SSP-RK3   0.97   1.03   1.18   1.15   1.11   1.17   1.09   1.03
+//   P^2 RK4       0.89   0.91   1.06   1.04   1.02   1.10   1.06   1.01
+//   Q^2 SSP-RK3   0.83   0.89   1.02   1.03   1.11   1.08   1.05   1.00
+//   Q^2 RK4       0.75   0.80   0.95   0.98   1.04   1.03   1.03   1.00
+//   P^3 SSP-RK3   0.67   0.65   0.83   0.93   0.97   0.97   0.99   0.97
+// advection in quadrature form (a row is a quarter of the work):
+//   Q^2 SSP-RK3   1.10   1.03   1.04   1.11   1.06   1.08   1.06   1.04
+//   Q^2 RK4       0.98   0.93   0.93   1.01   0.99   1.01   1.00   1.02
+//   P^3 RK4       0.94   0.85   0.79   0.91   0.87   0.91   0.95   0.99
+// Q^3 keeps tables on the stack: a row costs ten times P^3's (RK4, 96 x 96: 3.0 ms
+// with halo rows, 1.0 with seams).  Segments of one row in many waves (a launch
+// shape set so) are bound by the work, of which halo rows are two thirds: P^2
+// SSP-RK3 on 1920 x 480, 4 steps 2.28 / 1.72 ms (2 rows 1.58 / 1.62).
+inline bool use_seams(size_t esize, int stages, int modes, int nq, int nv, bool dev, bool lim_on_load, int ny, int n_segs,
+                      long long warps, int sms) {
     if (esize == 8) return true;
-    const int rows = stages * modes >= 27 ? (dev ? 64 : 6) : (stages * modes >= 18 ? 1 : 0);
-    return !lim_on_load && ny <= (long long)rows * n_segs;
+    if (lim_on_load) return false;
+    const int stage = modes * (nq * nq + 4 * nq), row = stages * stage;
+    const bool one = ny <= n_segs;   // a row a segment
+    if (stage >= 500 || row >= (nv == 1 ? 1200 : 900)) return true;
+    if (row >= 700) return nv == 1 ? one : ny <= (dev ? 3LL : 6LL) * n_segs;
+    if (nv > 1 && row >= 500 && one) return dev || warps >= 4LL * sms;
+    return nv > 1 && row >= 350 && one && warps >= 32LL * sms;
 }
 // What the seam scratch may take: an eighth of a state copy, or 256 MiB.  A launch
 // shape asks for memory in proportion to its segments, which seam_segments keeps
