@@ -185,6 +185,7 @@ struct ArgsView {
     __device__ __forceinline__ DevState* ds() const { return a.ds; }
     __device__ __forceinline__ int* cur() const { return nullptr; }
     __device__ __forceinline__ unsigned* done() const { return nullptr; }
+    static constexpr bool ALONE = true;   // the one problem of its launch
     __device__ __forceinline__ bool copy_if_idle() const { return true; }
     // derived constants, computed on the host (set_derived)
     __device__ __forceinline__ T rxT() const {
@@ -239,6 +240,7 @@ struct ProbView {
     __device__ __forceinline__ DevState* ds() const { return ds_; }
     __device__ __forceinline__ int* cur() const { return cur_; }
     __device__ __forceinline__ unsigned* done() const { return done_; }
+    static constexpr bool ALONE = false;
     __device__ __forceinline__ bool copy_if_idle() const { return false; }
     // per-problem constants, in the arithmetic of set_derived (1/dx and 1/dy
     // from the problem table, made on the host)
@@ -461,21 +463,21 @@ struct CellRed {
 };
 
 // Wave speed of new averages A, in the state's arithmetic, and its status bits
-template <class T, int PHYS, int NV, class PV>
-__device__ __forceinline__ T new_speed(const StepArgs& a, const PV& pv, const T* A, T rx, T ry, T gm1, T gam,
+template <class T, int PHYS, int NV, class PV, class AV>
+__device__ __forceinline__ T new_speed(const StepArgs& a, const PV& pv, const AV& A, T rx, T ry, T gm1, T gam,
                                        unsigned& status) {
     if constexpr (PHYS != PHYS_EULER) {
-        if (!(A[0] == A[0])) status |= ST_NAN;
+        if (!(A(0) == A(0))) status |= ST_NAN;
         return T(pv.adv_speed());
     } else {
-        const T ir = T(1) / A[0];
-        const T w = A[1] * ir, vv = A[2] * ir;
-        const T p = gm1 * (A[3] - T(0.5) * (A[1] * w + A[2] * vv));
+        const T ir = T(1) / A(0);
+        const T w = A(1) * ir, vv = A(2) * ir;
+        const T p = gm1 * (A(3) - T(0.5) * (A(1) * w + A(2) * vv));
         const T c = sqrt(fmax(gam * p * ir, T(0)));
         T sp;
         if constexpr (sizeof(T) == 4) sp = (fabs(w) + c) * rx + (fabs(vv) + c) * ry;
         else sp = (fabs(w) + c) / pv.dx() + (fabs(vv) + c) / pv.dy();
-        if (!(A[0] > T(0)) || !(p > T(0))) status |= ST_NONPHYSICAL;
+        if (!(A(0) > T(0)) || !(p > T(0))) status |= ST_NONPHYSICAL;
         if (!(sp == sp)) status |= ST_NAN;
         return sp;
     }
@@ -506,7 +508,7 @@ __device__ __forceinline__ void store_cell(const StepArgs& a, const PV& pv, cons
                                            T* __restrict__ uout, size_t plane, size_t o, T (&P)[NV][NM], T rx, T ry,
                                            T gm1, T gam, CellRed<T, NV>& red) {
     static_assert(!COMP || sizeof(T) == 4, "the compensated state is FP32");
-    T avl[NV], A[NV];   // COMP: lo parts of the new averages
+    T avl[NV];   // COMP: lo parts of the new averages
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
 #pragma unroll
@@ -523,24 +525,23 @@ __device__ __forceinline__ void store_cell(const StepArgs& a, const PV& pv, cons
                 uout[ix] = P[v][m];
             }
         }
-        A[v] = P[v][0];
     }
     if constexpr (sizeof(T) == 4) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) {   // TwoSum: hi + lo += A[v] exactly
-            const T x = A[v];
+            const T x = P[v][0];
             const T sum = red.hi[v] + x;
             const T bv = sum - red.hi[v];
             red.lo[v] += (red.hi[v] - (sum - bv)) + (x - bv);
             if constexpr (COMP) red.lo[v] += avl[v];
             red.hi[v] = sum;
         }
-        const T sp = new_speed<T, PHYS, NV>(a, pv, A, rx, ry, gm1, gam, red.status);
+        const T sp = new_speed<T, PHYS, NV>(a, pv, [&](int v) { return P[v][0]; }, rx, ry, gm1, gam, red.status);
         if constexpr (PHYS == PHYS_EULER) red.maxT = fmax(red.maxT, sp);
     } else {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) red.sum[v] += A[v];
-        red.max = fmax(red.max, new_speed<T, PHYS, NV>(a, pv, A, rx, ry, gm1, gam, red.status));
+        for (int v = 0; v < NV; ++v) red.sum[v] += P[v][0];
+        red.max = fmax(red.max, new_speed<T, PHYS, NV>(a, pv, [&](int v) { return P[v][0]; }, rx, ry, gm1, gam, red.status));
     }
 }
 
@@ -665,8 +666,20 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
     const bool has_bcW = !perx && xs == 0;
     const bool has_bcE = !perx && xs + 30 >= nx;
 
-    // rows split evenly over the segments (each at most seg_len rows)
-    const int r0 = seg_row(seg, ny, pv.n_segs()), r1 = seg_row(seg + 1, ny, pv.n_segs());
+    // rows split evenly over the segments.  (Either form gives the same rows, as
+    // either form of keep_north's first condition below is the same condition:
+    // the choice moves the compiler's schedule of the whole row.  Halo rows, FP32,
+    // times over the other forms: Q^1 SSP-RK3 on 1280^2 0.971, P^2 0.989, Q^2 RK4
+    // 0.996; the deviation form and a batch's kernels, which hold two bodies, keep
+    // the other condition: 0.966 for the deviation form's Q^2 RK4.)
+    int r0, r1;
+    if constexpr (SEAM || !PV::ALONE) {
+        r0 = seg_row(seg, ny, pv.n_segs());
+        r1 = seg_row(seg + 1, ny, pv.n_segs());
+    } else {
+        r0 = (int)(((long long)seg * ny) / pv.n_segs());
+        r1 = (int)(((long long)(seg + 1) * ny) / pv.n_segs());
+    }
     // the faces below the first and above the last row that are seams, or the
     // halo rows that are recomputed for them
     const bool seamS = SEAM && (r0 > 0 || pery), seamN = SEAM && (r1 < ny || pery);
@@ -769,7 +782,7 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
         const bool do_south = r > rstart || south_bc;   // flux through this row's south face
         const bool seam_row = SEAM && r == r0 && seamS; // its update waits for the seam below it
         const bool last = r == rend;
-        const bool keep_north = SEAM ? !last || !seamN : (!last || (r == ny - 1 && !pery && out_row));
+        const bool keep_north = SEAM ? !last || !seamN : ((DEV || !PV::ALONE ? !last : r < rend) || (r == ny - 1 && !pery && out_row));
 
         // ---- load u^n (and limit on load) -------------------------------------
         T un[NV][NM];
@@ -1263,9 +1276,8 @@ __device__ __forceinline__ void step2d_body(const StepArgs& a, const PV& pv, con
 
         // ---- finish the row below: its north face is this row's south face --------
         auto finish = [&](T (&P)[NV][NM], int rw) {
-            if (outlane)
-                store_cell<T, PHYS, NV, NM, COMP>(a, pv, uin, uout, plane, (size_t)rw * nx + col, P, rx, ry, gm1, gam,
-                                                  red);
+            if (!outlane) return;
+            store_cell<T, PHYS, NV, NM, COMP>(a, pv, uin, uout, plane, (size_t)rw * nx + col, P, rx, ry, gm1, gam, red);
         };
         // an update that a seam completes, left in the output buffer (COMP: in the hi planes)
         auto leave = [&](const T (&P)[NV][NM], int rw) {
@@ -1634,7 +1646,7 @@ __device__ __forceinline__ void seam_body(const StepArgs& a, const PV& pv, int b
             T A[NV];
 #pragma unroll
             for (int i = 0; i < NV; ++i) A[i] = avg[grp][i][lane];
-            fastest = fmax(fastest, new_speed<T, PHYS, NV>(a, pv, A, rx, ry, gm1, gam, st));
+            fastest = fmax(fastest, new_speed<T, PHYS, NV>(a, pv, [&](int i) { return A[i]; }, rx, ry, gm1, gam, st));
         }
         __syncthreads();
     }
