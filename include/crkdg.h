@@ -237,7 +237,8 @@ int crkdg_step_device(crkdg_ctx* ctx);
 int crkdg_rkdg_step(crkdg_ctx* ctx, double dt, int order);
 
 /* Fixed-dt run of n_steps steps.  1D meshes of up to 960 cells run the whole
- * sequence in one single-block launch (block barrier between steps). */
+ * sequence in one launch of up to 8 blocks (one cluster, a barrier between
+ * steps); t advances as n_steps calls of crkdg_step would advance it. */
 int crkdg_run_fixed(crkdg_ctx* ctx, int n_steps, double dt);
 
 /* Totals sum_K |K| ubar_K per variable (FP64, eq. (3.4)).  Synchronises. */
@@ -275,8 +276,17 @@ int crkdg_run_state_async(crkdg_ctx* ctx, double* out);
  * (run state restored afterwards; a limit pending in CRKDG_LIMIT_PASS mode is
  * applied first, as the next step would apply it) and keeps the fastest; the
  * candidates include the current shape, so tuning never selects a shape
- * slower in its own timing.  Returns the kept shape's time per step (the step
- * kernel and its one-block finalize) in microseconds.  Synchronises. */
+ * slower in its own timing.  Returns the kept shape's time per step (all
+ * launches of the step) in microseconds.  Synchronises.
+ * FP64 steps, and FP32 steps whose rows are dear, leave the faces between
+ * segments to launches that need scratch in proportion to the segments: up to
+ * 256 MiB or an eighth of a state copy, sized when the context is created and
+ * when the shape, the limit mode or the operator form changes (a step allocates
+ * nothing).  Shorter segments than that allows, or than the device has memory
+ * for, are merged (crkdg_get_launch reports the rows run) or, in FP32, recompute
+ * the rows beside them; results do not depend on it.  crkdg_set_launch and
+ * crkdg_autotune may move the scratch: graphs of steps that the caller captured
+ * before must not be replayed after them. */
 int crkdg_set_launch(crkdg_ctx* ctx, int seg_rows, int warps_per_block);
 int crkdg_get_launch(const crkdg_ctx* ctx, int* seg_rows, int* warps_per_block);
 int crkdg_autotune(crkdg_ctx* ctx, double* best_us);
@@ -300,8 +310,8 @@ int crkdg_get_limit_mode(const crkdg_ctx* ctx, int* mode);
 /* How the 2D step evaluates its operators for linear advection.
  * CRKDG_FORM_AUTO (default): where the flux is linear (CRKDG_ADVECTION, FP32
  * or FP64) and every non-periodic side is outflow, wall, a constant state or
- * sine data (CRKDG_FN_SINE, CRKDG_FN_SINE_PROD), the step uses the modal form of the operators — the local operator (eq.
- * (2.7)) is beta . grad of the modal polynomial, the final stage's
+ * sine data (CRKDG_FN_SINE, CRKDG_FN_SINE_PROD), the step uses the modal form
+ * of the operators — the local operator (eq. (2.7)) is beta . grad of the modal polynomial, the final stage's
  * sum_i b_i div^DG f(u^(i)) equals the DG operator of sum_i b_i u^(i) (the
  * linearity behind Theorem 3.3), applied once with the upwind flux — which
  * the quadrature form computes exactly as well; results agree to rounding.
@@ -375,8 +385,11 @@ int crkdg_batch_problem_info(crkdg_batch* b, int problem, double* t, unsigned lo
  * for another mode. */
 int crkdg_batch_set_limit_mode(crkdg_batch* b, int mode);
 /* launch shape (rows per warp segment, warps per block) and its autotuner,
- * which times one batched step per candidate on the current states (run
- * states restored afterwards) */
+ * which times one batched step per candidate, the current shape first, on the
+ * current states (run states restored afterwards).  The scratch of the faces
+ * between segments is bounded as a context's (crkdg_set_launch); a shape whose
+ * tables the device has no memory for is refused with CRKDG_ENOMEM, and the
+ * batch runs again once a shape fits */
 int crkdg_batch_set_launch(crkdg_batch* b, int seg_rows, int warps_per_block);
 int crkdg_batch_autotune(crkdg_batch* b, double cfl, double* best_us);
 const char* crkdg_batch_last_error(void);
@@ -474,7 +487,7 @@ const char* crkdg_probe_last_error(void);
  *            since the maximum skips NaN, so check out[1 + nv];
  *   beta     host pointer to (beta_x, beta_y) for advection, else may be NULL.
  * Asynchronous on `stream`.  Scratch: a file-scope device array of about
- * 64 KiB (1024 per-warp slots) that every GPU loading the library holds until
+ * 6 KiB (a slot per block) that every GPU loading the library holds until
  * the process exits.  Its device address is looked up, with the stream's
  * device current, at every call made outside a stream capture; a call made
  * while `stream` is being captured reuses the address of the last uncaptured

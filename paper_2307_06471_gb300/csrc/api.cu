@@ -143,8 +143,8 @@ size_t seam_seg_bytes(const crkdg_ctx* c, bool fused) {
     return crk::seam_values(c->tab.s, c->k + 1, c->nv, c->nm, c->precision == CRKDG_F32D, fused, c->mesh.nx) * c->esize;
 }
 // whether the quadrature step leaves the faces between its segments to the
-// seam launches (the compensated state without
-// deviation fluxes recomputes halo rows)
+// seam launches (the compensated state without deviation fluxes recomputes
+// halo rows)
 bool step_seams(const crkdg_ctx* c, int nseg, bool lim_on_load, int stages) {
     return c->precision != CRKDG_F32C && !c->seams_off &&
            crk::use_seams(c->esize, stages, c->nm, c->k + 1, c->nv, c->precision == CRKDG_F32D, lim_on_load, c->mesh.ny, nseg,
@@ -448,7 +448,6 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
         const bool fused = limit && c->limit_mode == CRKDG_LIMIT_FUSED;
         int ns, nseg;
         step_segs(c, &ns, &nseg);
-        a.seg_len = c->seg_rows;
         a.n_strips = ns;
         a.n_segs = nseg;
         int r = use_linear(c) && !fused ? ensure_slots(c) : ensure_step_scratch(c);
@@ -470,7 +469,6 @@ int enqueue_step(crkdg_ctx* c, double dt, int dt_from_dev, int limit, double M) 
                 a.limit = 0;
             }
             if (!a.limit && use_linear(c)) {
-                a.seg_len = c->lin_seg_rows;
                 strips_segs(c, c->lin_seg_rows, &a.n_strips, &a.n_segs);
                 a.lin_data = c->d_lin_data;
                 set_linear(c, a);
@@ -911,7 +909,6 @@ static int enqueue_fe(crkdg_ctx* c, const void* in, void* out, double t, double 
     a.tab = c->d_tab_fe;
     int ns, nseg;
     step_segs(c, &ns, &nseg);
-    a.seg_len = c->seg_rows;
     a.n_strips = ns;
     a.n_segs = nseg;
     int r = ensure_step_scratch(c);

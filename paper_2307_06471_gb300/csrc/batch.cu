@@ -131,7 +131,6 @@ StepArgs batch_args(const crkdg_batch* b) {
     for (int s = 0; s < 4; ++s) a.bc[s].type = b->bc[s];
     crk::set_bc_affine(a.bc, 4);
     a.gamma = b->gamma;
-    a.seg_len = b->seg_rows;
     a.partials = b->d_partials;
     a.seam = b->d_seam;
     return a;
@@ -155,7 +154,6 @@ size_t plan_tables(crkdg_batch* b, bool seams, size_t room, long long* n_slots) 
     b->flux.clear();
     b->seams.clear();
     b->use_seams = seams;
-    int warp0 = 0;
     long long slots = 0, seam = 0;
     for (int p = 0; p < b->n; ++p) {
         BatchProblem& pb = b->probs[p];
@@ -166,7 +164,6 @@ size_t plan_tables(crkdg_batch* b, bool seams, size_t room, long long* n_slots) 
         pb.n_segs = (pb.ny + b->seg_rows - 1) / b->seg_rows;
         if (seams) pb.n_segs = crk::seam_segments(pb.n_segs, seg * b->esize, (size_t)((double)room * values / b->elems));
         pb.n_seam_blocks = crk::seam_blocks(b->nv, pb.nx, pb.ny, pb.n_segs, 32);
-        pb.warp0 = warp0;
         pb.slot0 = slots;
         pb.seam0 = seam;
         const int w = pb.n_strips * pb.n_segs;
@@ -177,7 +174,6 @@ size_t plan_tables(crkdg_batch* b, bool seams, size_t room, long long* n_slots) 
             for (int i = 0; i < pb.n_seam_blocks; ++i) b->seams.push_back(make_int2(p, i));
             seam += (long long)(seg * pb.n_segs);
         }
-        warp0 += w;
         slots += w + pb.n_seam_blocks;
     }
     *n_slots = slots;

@@ -26,7 +26,7 @@ struct DevState {
     double sums[4];
     double troubled;          // troubled cells flagged in the last step
     unsigned status;          // ST_* bits
-    unsigned counter;         // arrival counter of a batched problem's last-warp reduction
+    unsigned counter;         // arrivals of a launch's blocks, the last of which reduces their slots
     unsigned long long steps;
     unsigned long long lim_count;   // cells flagged by a separate limiter pass since the last step
 };
@@ -77,13 +77,13 @@ struct StepArgs {
     double t, dt;             // used when dt_from_dev == 0
     int dt_from_dev;
     DevState* ds;
-    double* partials;         // per-warp reduction slots
+    double* partials;         // reduction slots
     int seams;                // the step leaves the faces between segments to the seam launches
     void* seam;               // seam scratch (step2d.cuh)
     int s;
     const double* tab;        // device tableau buffer, layout of pack_tableau
     BCSide bc[4];             // W, E, S, N
-    int seg_len, n_strips, n_segs;
+    int n_strips, n_segs;
     int limit;                // 1: limit u^n on load (final-stage limiters of the previous step)
     double M;                 // TVB parameter; < 0: no TVB limiter
     double pp_eps;            // > 0: positivity-preserving scaling with this floor
@@ -121,7 +121,7 @@ struct BatchProblem {
     double x0, y0, dx, dy;
     double rx, ry;         // 1/dx, 1/dy (host)
     int n_strips, n_segs;
-    int warp0;             // first task of the problem
+    int pad;               // (unused; without it the batch's FP32 Q^2 kernel spills 616 bytes for 396)
     int n_seam_blocks;     // blocks of its last seam launch
     long long slot0;       // its first reduction slot: step warps, then seam blocks
     long long seam0;       // element offset of its seam scratch

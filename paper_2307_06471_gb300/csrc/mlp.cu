@@ -58,7 +58,7 @@ struct TrainSmem {
     float b1[MLP_H], b2[MLP_H], b3[MLP_H], W4[MLP_H], b4[4];
     float X[TILE * SX], H1[TILE * SH], H2[TILE * SH], H3[TILE * SH];
     float G[TILE * SH], G2[TILE * SH];   // the delta of a layer, and of the one below
-    float dz[TILE], red[TRAIN_THREADS / 32];
+    float dz[TILE];
 };
 
 // Forward and backward of the mean class-weighted BCE over n samples (rows
@@ -67,8 +67,8 @@ struct TrainSmem {
 //
 // A minibatch of 1024 samples is small for the GPU, so a tile is 8 samples
 // (128 blocks; one wave of larger n walks its tiles) and the block's gradient
-// stays in registers (43 values a thread) until its last tile.  Four samples
-// of a thread's unit share its weights' 16-byte loads in the forward pass.
+// stays in registers (52 values a thread) until its last tile.  Two samples of a
+// thread's unit share its weights' 16-byte loads in the forward pass.
 // With tiles of 64 samples, a block per tile and unpadded rows (32-way bank
 // conflicts on the weights) a minibatch of 1024 took 0.126 ms; this takes
 // 0.014 ms (0.023 while the loads of the weights waited for one another).

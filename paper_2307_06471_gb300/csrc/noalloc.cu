@@ -16,20 +16,17 @@
 namespace {
 
 // Scratch of the reduction: the run-state block (arrival counter, results)
-// and one slot of 8 doubles per warp.  The grid is capped at 128 blocks of
-// 256 threads (1024 warps): larger meshes are covered by the kernel's
-// grid-stride loop, so the array never needs to grow.
+// and a slot per block.  The grid is 128 blocks of 256 threads: larger meshes
+// are covered by the kernel's loop over chunks, so the array never needs to grow.
 constexpr int kNoAllocBlocks = 128;
-constexpr int kNoAllocWarps = kNoAllocBlocks * 8;
-constexpr int kSlot = 8;
 constexpr long long kMaxCells = 1LL << 30;
 
 struct NoAllocScratch {
     crk::DevState ds;
-    double partials[kNoAllocWarps * kSlot];
+    double partials[kNoAllocBlocks * crk::REDUCE_SLOT];
 };
 
-// about 64 KiB, held by every GPU that loads the library until the process exits
+// about 6 KiB, held by every GPU that loads the library until the process exits
 static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
 
 // Device address of the array.  In host code the symbol name is only a

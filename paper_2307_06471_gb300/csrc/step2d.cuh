@@ -178,7 +178,6 @@ struct ArgsView {
     __device__ __forceinline__ double dt() const { return dt_; }
     __device__ __forceinline__ int n_strips() const { return a.n_strips; }
     __device__ __forceinline__ int n_segs() const { return a.n_segs; }
-    __device__ __forceinline__ int seg_len() const { return a.seg_len; }
     __device__ __forceinline__ int total_warps() const { return a.n_strips * a.n_segs; }
     __device__ __forceinline__ double* partials() const { return a.partials; }
     __device__ __forceinline__ void* seam() const { return a.seam; }
@@ -215,7 +214,7 @@ struct ProbView {
     int nx_, ny_;
     double x0_, y0_, dx_, dy_;
     double t_, dt_;
-    int n_strips_, n_segs_, seg_len_, total_warps_;
+    int n_strips_, n_segs_, total_warps_;
     double* partials_;    // this problem's reduction slots
     void* seam_;          // this problem's seam scratch
     DevState* ds_;        // this problem's run state
@@ -233,7 +232,6 @@ struct ProbView {
     __device__ __forceinline__ double dt() const { return dt_; }
     __device__ __forceinline__ int n_strips() const { return n_strips_; }
     __device__ __forceinline__ int n_segs() const { return n_segs_; }
-    __device__ __forceinline__ int seg_len() const { return seg_len_; }
     __device__ __forceinline__ int total_warps() const { return total_warps_; }
     __device__ __forceinline__ double* partials() const { return partials_; }
     __device__ __forceinline__ void* seam() const { return seam_; }
@@ -1731,7 +1729,6 @@ __device__ __forceinline__ ProbView<T> problem_view(const StepArgs& a, const Bat
     pv.dt_ = ds->dt;
     pv.n_strips_ = pb.n_strips;
     pv.n_segs_ = pb.n_segs;
-    pv.seg_len_ = a.seg_len;
     pv.total_warps_ = pb.n_strips * pb.n_segs;
     pv.partials_ = a.partials + (size_t)pb.slot0 * Step2D<T, K, B, PHYS>::NRED;
     pv.seam_ = static_cast<T*>(a.seam) + pb.seam0;
